@@ -273,6 +273,18 @@ __device__ __forceinline__ void store_words(const AdjArgs &a, uint4 *wp, int64_t
     }
 }
 
+// Counter block m of the thread's two trajectories.  They share the block's head unless
+// their global ids differ in the high word (a pair astride a multiple of 2^32, only for
+// some traj_base): then the second one's is formed on its own.
+__device__ __forceinline__ void pair_blocks(uint32_t m, const StepStream (&ss)[2], const RoundKeys &K, uint4 &w0,
+                                            uint4 &w1) {
+    const BlockHead h0 = block_head(m, ss[0].hx);
+    BlockHead h1 = h0;
+    if (ss[1].hx != ss[0].hx) h1 = block_head(m, ss[1].hx);
+    w0 = step_block(h0, ss[0], K);
+    w1 = step_block(h1, ss[1], K);
+}
+
 template <bool WORDS>
 __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<float> &k, const StepStream (&ss)[2],
                                                 const int64_t (&idx)[2], bool store1, int64_t s0, int64_t s1,
@@ -305,7 +317,8 @@ __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<flo
 #pragma unroll
                 for (int b2 = 0; b2 < kSub / 4; ++b2) {
                     const uint32_t m = (uint32_t)(n0 >> 2) + b2;
-                    const uint4 w0 = step_block(m, ss[0], a.K), w1 = step_block(m, ss[1], a.K);
+                    uint4 w0, w1;
+                    pair_blocks(m, ss, a.K, w0, w1);
                     float2 nrA, nrB, cs, sn;
                     box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nrA, cs, sn);
                     em_step_f32x2(k2, nrA, cs, PB, Y, V, E);
@@ -345,7 +358,8 @@ __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<flo
 #pragma unroll
             for (int b2 = 0; b2 < kSub / 4; ++b2) {
                 const uint32_t m = (uint32_t)(n0 >> 2) + b2;
-                const uint4 w0 = step_block(m, ss[0], a.K), w1 = step_block(m, ss[1], a.K);
+                uint4 w0, w1;
+                pair_blocks(m, ss, a.K, w0, w1);
                 float2 nrA, nrB, cs, sn;
                 box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nrA, cs, sn);
                 em_step_f32x2(k2, nrA, cs, PB, Y, V, E);
@@ -560,7 +574,8 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
                     tr[3] = sn;
                 } else {
                     const uint32_t m = (uint32_t)(n0 >> 2) + b2;
-                    const uint4 w0 = step_block(m, ss[0], a.K), w1 = step_block(m, ss[1], a.K);
+                    uint4 w0, w1;
+                    pair_blocks(m, ss, a.K, w0, w1);
                     box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nr[0], cs, sn);
                     tr[0] = cs;
                     tr[1] = sn;

@@ -59,45 +59,48 @@ struct RoundKeys {
 };
 
 // The step noise of one trajectory: counter (m, 0, t_lo, t_hi) for m < 2^32.
-// The first round's products with the trajectory words do not depend on m
-// and are formed once per trajectory (pre0 = hi(M1 t_lo) ^ k0, pre1 = lo(M1 t_lo)).
+// Rounds 0 and 1 separate: after round 0 the words are (hi(M1 t_lo) ^ k0, lo(M1 t_lo),
+// hi(M0 m) ^ t_hi ^ k1, lo(M0 m)), so round 1's product by M0 is the trajectory's own
+// and its product by M1 depends on (m, t_hi) alone.  StepStream keeps the first,
+// formed once per trajectory; BlockHead is the second, formed once per counter block
+// for every trajectory of a thread that shares t_hi.  A block of two trajectories
+// takes 34 wide multiplies (2 shared, 16 each) instead of 37.
 struct StepStream {
-    uint32_t pre0, pre1, c3x;  // c3x = t_hi ^ k1 of round 0
+    uint32_t a, b, c;  // lo(M1 t_lo) ^ rk[2], hi(p) ^ rk[3], lo(p), p = M0 (hi(M1 t_lo) ^ rk[0])
+    uint32_t hx;       // t_hi ^ rk[1]
+};
+struct BlockHead {
+    uint32_t u0, u1, u2;  // hi(q), lo(q), lo(M0 m), q = M1 (hi(M0 m) ^ hx)
 };
 
 __device__ __forceinline__ StepStream step_stream(uint64_t t, const RoundKeys &K) {
     StepStream s;
     const uint32_t tlo = (uint32_t)t, thi = (uint32_t)(t >> 32);
     const uint64_t p1 = (uint64_t)kPhiloxM1 * tlo;
-    s.pre0 = (uint32_t)(p1 >> 32) ^ K.rk[0];  // c1 = m_hi = 0
-    s.pre1 = (uint32_t)p1;
-    s.c3x = thi ^ K.rk[1];
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * ((uint32_t)(p1 >> 32) ^ K.rk[0]);  // c1 = m_hi = 0
+    s.a = (uint32_t)p1 ^ K.rk[2];
+    s.b = (uint32_t)(p0 >> 32) ^ K.rk[3];
+    s.c = (uint32_t)p0;
+    s.hx = thi ^ K.rk[1];
     return s;
 }
 
-#ifndef ABP_KEYS_IN_KERNEL
-#define ABP_KEYS_IN_KERNEL 0
-#endif
+__device__ __forceinline__ BlockHead block_head(uint32_t m, uint32_t hx) {
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * m;
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * ((uint32_t)(p0 >> 32) ^ hx);
+    return BlockHead{(uint32_t)(p1 >> 32), (uint32_t)p1, (uint32_t)p0};
+}
+
+// Rounds 2..9 of one trajectory's counter block, from the block's head.
+__device__ __forceinline__ uint4 step_block(const BlockHead &h, const StepStream &s, const RoundKeys &K) {
+    uint32_t c0 = h.u0 ^ s.a, c1 = h.u1, c2 = h.u2 ^ s.b, c3 = s.c;
+#pragma unroll
+    for (int r = 2; r < 10; ++r) philox_round(c0, c1, c2, c3, K.rk[2 * r], K.rk[2 * r + 1]);
+    return make_uint4(c0, c1, c2, c3);
+}
 
 __device__ __forceinline__ uint4 step_block(uint32_t m, const StepStream &s, const RoundKeys &K) {
-    // round 0 with the trajectory half precomputed
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * m;
-    uint32_t c0 = s.pre0, c1 = s.pre1;
-    uint32_t c2 = (uint32_t)(p0 >> 32) ^ s.c3x;
-    uint32_t c3 = (uint32_t)p0;
-#if ABP_KEYS_IN_KERNEL
-    uint32_t k0 = K.rk[0], k1 = K.rk[1];
-#pragma unroll
-    for (int r = 1; r < 10; ++r) {
-        k0 += kPhiloxW0;
-        k1 += kPhiloxW1;
-        philox_round(c0, c1, c2, c3, k0, k1);
-    }
-#else
-#pragma unroll
-    for (int r = 1; r < 10; ++r) philox_round(c0, c1, c2, c3, K.rk[2 * r], K.rk[2 * r + 1]);
-#endif
-    return make_uint4(c0, c1, c2, c3);
+    return step_block(block_head(m, s.hx), s, K);
 }
 
 // Counter of the initial-condition draw (m = 2^63; step counters stay below 2^32).
@@ -127,7 +130,16 @@ __device__ __forceinline__ uint4 xorshift_seed(uint64_t t, uint32_t k0, uint32_t
 
 // --------------------------------------------------------------------------
 // Hardware approximations used by the FP32 path.  The approximate square
-// root is the PTX instruction itself; log2 and sin/cos are CUDA's intrinsics.
+// root and log2 are the PTX instructions themselves; sin/cos are CUDA's intrinsics.
+// log2: __log2f without -ftz also rescales subnormal arguments (three more
+// instructions per call); the argument here is a u1 >= 2^-33, never subnormal, so the
+// flushing form returns the same value.
+__device__ __forceinline__ float log2_approx(float x) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
 __device__ __forceinline__ float sqrt_approx(float x) {
     float r;
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -142,6 +154,10 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr float kTwoPiF = 6.28318530717958647692f;
 constexpr float kLn2F = 0.69314718055994530942f;
 
+// 1 + floor(w / 2^9) 2^-23: the top 23 bits of w as the mantissa of a float in [1, 2)
+// (one funnel shift that brings the exponent bits in from above).
+__device__ __forceinline__ float unit_mantissa(uint32_t w) { return __uint_as_float(__funnelshift_r(w, 127u, 9)); }
+
 // Box-Muller of one word pair, FP32.  u1 = (wa + 1/2) 2^-32 (I2F rounds to
 // nearest, the fused multiply-add adds the half exactly), u2 = floor(wb/2^9)
 // 2^-23 built from the top 23 bits as f = 1 + u2 in [1, 2).  The angle is
@@ -152,9 +168,9 @@ constexpr float kLn2F = 0.69314718055994530942f;
 __device__ __forceinline__ void box_muller_f32(uint32_t wa, uint32_t wb, float c2, float &nrs, float &cs,
                                                float &sn) {
     const float u1 = fmaf(__uint2float_rn(wa), 0x1p-32f, 0x1p-33f);
-    const float l2 = __log2f(u1);  // <= 0
+    const float l2 = log2_approx(u1);  // <= 0
     nrs = -sqrt_approx(fabsf(l2 * c2));
-    const float f = __uint_as_float(0x3f800000u | (wb >> 9));
+    const float f = unit_mantissa(wb);
 #if ABP_ANGLE_FFMA
     __sincosf(fmaf(f, kTwoPiF, -1.5f * kTwoPiF), &sn, &cs);
 #else
@@ -360,12 +376,12 @@ __device__ __forceinline__ Coef2 make_coef2(const Coef<float> &k) {
 __device__ __forceinline__ float2 bm_radius_f32x2(uint2 wa, float2 c2) {
     const float2 u1 =
         __ffma2_rn(make_float2(__uint2float_rn(wa.x), __uint2float_rn(wa.y)), dup2(0x1p-32f), dup2(0x1p-33f));
-    const float2 p = __fmul2_rn(make_float2(__log2f(u1.x), __log2f(u1.y)), c2);
+    const float2 p = __fmul2_rn(make_float2(log2_approx(u1.x), log2_approx(u1.y)), c2);
     return make_float2(-sqrt_approx(fabsf(p.x)), -sqrt_approx(fabsf(p.y)));
 }
 
 __device__ __forceinline__ void bm_angle_f32x2(uint2 wb, float2 &cs, float2 &sn) {
-    const float2 f = make_float2(__uint_as_float(0x3f800000u | (wb.x >> 9)), __uint_as_float(0x3f800000u | (wb.y >> 9)));
+    const float2 f = make_float2(unit_mantissa(wb.x), unit_mantissa(wb.y));
     const float2 ang = __ffma2_rn(f, dup2(kTwoPiF), dup2(-1.5f * kTwoPiF));
     __sincosf(ang.x, &sn.x, &cs.x);
     __sincosf(ang.y, &sn.y, &cs.y);

@@ -18,24 +18,14 @@
 #include "abp_device.cuh"
 #include "abp_internal.cuh"
 
-// Minimum resident blocks per SM requested from the compiler for the
-// integrator (bounds its register use); 0 leaves the choice to the compiler.
 // Counter blocks (4 steps each) per iteration of the integrator's inner loop.
 #ifndef ABP_GROUP_UNROLL
-#define ABP_GROUP_UNROLL 2
+#define ABP_GROUP_UNROLL 4
 #endif
 // Warp-specialised narrow launches (noise drawn by producer warps); 0 keeps
 // every narrow launch on the plain integrator.
 #ifndef ABP_WS
 #define ABP_WS 1
-#endif
-#ifndef ABP_MIN_BLOCKS
-#define ABP_MIN_BLOCKS 0
-#endif
-#if ABP_MIN_BLOCKS > 0
-#define ABP_INTEGRATE_BOUNDS __launch_bounds__(abp::kThreads, ABP_MIN_BLOCKS)
-#else
-#define ABP_INTEGRATE_BOUNDS __launch_bounds__(abp::kThreads)
 #endif
 
 namespace abp {
@@ -246,7 +236,7 @@ constexpr bool kPaired = sizeof(R) == 4 && PPT % 2 == 0 && ABP_F32X2 && ABP_ANGL
 // One Euler-Maruyama step of every slot at an arbitrary step index n (the
 // unaligned head / tail of a range): the counter block of n is generated for
 // this step alone.
-template <typename R, int PPT, int MODE = kModeEM>
+template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true>
 __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, int64_t n) {
     if constexpr (MODE == kModeXorshift && kPaired<R, PPT>) {
         const Coef2 k2 = make_coef2(k);
@@ -276,10 +266,10 @@ __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K
         return;
     }
     const uint32_t j = (uint32_t)(n & 3);
-    const uint32_t m = (uint32_t)(n >> 2);
+    const BlockHead head = block_head((uint32_t)(n >> 2), S.ss[0].hx);
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
-        const uint4 w = step_block(m, S.ss[q], K);
+        const uint4 w = SHARED ? step_block(head, S.ss[q], K) : step_block((uint32_t)(n >> 2), S.ss[q], K);
         if constexpr (sizeof(R) == 4) {
             float nrs, cs, sn;
             if (j < 2)
@@ -294,8 +284,9 @@ __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K
     }
 }
 
-// Four steps 4m .. 4m+3 of every slot from one counter block each.
-template <typename R, int PPT, int MODE = kModeEM>
+// Four steps 4m .. 4m+3 of every slot from one counter block each.  SHARED: the
+// slots' global ids have one high word, so one block head serves them all.
+template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true>
 __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, uint32_t m) {
     if constexpr (MODE == kModeXorshift) {
 #pragma unroll
@@ -303,9 +294,10 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
         return;
     }
     constexpr bool HEUN = MODE == kModeHeun;
+    const BlockHead head = block_head(m, S.ss[0].hx);
     uint4 w[PPT];
 #pragma unroll
-    for (int q = 0; q < PPT; ++q) w[q] = step_block(m, S.ss[q], K);
+    for (int q = 0; q < PPT; ++q) w[q] = SHARED ? step_block(head, S.ss[q], K) : step_block(m, S.ss[q], K);
     if constexpr (kPaired<R, PPT>) {
         // trajectories 2p and 2p + 1 in the two halves of FP32 register pairs
         const Coef2 k2 = make_coef2(k);
@@ -349,18 +341,17 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
     }
 }
 
-// Counter blocks per iteration of the inner loop, per kernel (measured): the
-// lockstep FP32 Euler-Maruyama kernel with two trajectories per thread runs
-// fastest with 8 blocks (32 steps) per iteration on the D x q sweep, 1.038e12
-// against 1.011e12 particle-steps/s with 2 and 0.98e12 with 12 (a body that no
-// longer fits the instruction cache).  The work-queue kernel takes 8 as well, at
-// 92 registers and two blocks per SM: against 6 (the same registers), uneven
-// batch 1.005e12 against 9.89e11, load sweep 9.95e11 against 9.83e11, D x q sweep
-// 1.020e12 against 1.006e12; capped at 80 registers for three blocks per SM it
-// spills and loses 8% on the load sweep.  The stochastic Heun kernel at two per
-// thread takes 4 (D x q sweep 6.92e11 against 6.88e11 with 2 and 3).  The other
-// kernels keep the default, where longer bodies cost registers and blocks per SM
-// without a measured gain.
+// Counter blocks per iteration of the inner loop, per kernel (measured on GB300,
+// D x q grids of 1,024 trajectories per set).  What bounds these loops is the FMA-heavy
+// pipe, 82% busy: a wide multiply of Philox holds it four cycles, a paired FP32
+// instruction two, and the two and the ALU's exclusive-ors do not overlap freely
+// (micro-benchmarks of the same mix reach 83-88%), so the body length decides how well
+// the compiler interleaves them.  FP32 Euler-Maruyama at two trajectories per thread
+// takes 8 blocks: 2,048 sets x 20,000 steps in 38.1 ms on the work queue (6: 39.4 ms, 10:
+// 38.9) and 38.5 ms lockstep.  Stochastic Heun takes 4 (512 sets x 10^4 steps 7.67 ms;
+// 2: 7.75, 3: 7.78, 6: 7.76), xorshift 8 (4.91 ms; 4: 4.93, 2: 5.04).  The other FP32
+// kernels take 4: one trajectory per thread 41.8 ms (2: 42.4, 1: 44.9), four 38.9 ms
+// (2: 40.2).  The FP64 kernels keep 2, longer bodies spill.
 #ifndef ABP_UNROLL_EM2
 #define ABP_UNROLL_EM2 8
 #endif
@@ -370,36 +361,56 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
 #ifndef ABP_UNROLL_HEUN2
 #define ABP_UNROLL_HEUN2 4
 #endif
+#ifndef ABP_UNROLL_XS2
+#define ABP_UNROLL_XS2 8
+#endif
 template <typename R, int PPT, int MODE, bool QUEUE>
 constexpr int group_unroll() {
     if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeEM)
         return QUEUE ? ABP_UNROLL_EM2_QUEUE : ABP_UNROLL_EM2;
     else if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeHeun)
         return ABP_UNROLL_HEUN2;
+    else if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift)
+        return ABP_UNROLL_XS2;
+    else if constexpr (sizeof(R) == 8)
+        return 2;
     else
         return kGroupUnroll;
 }
 
+// Resident blocks per SM asked of the compiler (bounds its registers; 0: its own choice).
+// The xorshift kernels at two trajectories per thread take four (64 registers, no
+// spills): 512 x 1,024 trajectories x 10^4 steps in 4.91 ms against 5.13 ms (work queue)
+// and 5.30 ms (lockstep) with three.  The others gain nothing from it (Euler-Maruyama
+// 38.4-39.3 ms against 38.0, Heun 7.80 against 7.65: not bound by latency).
+#ifndef ABP_BLOCKS_XS2
+#define ABP_BLOCKS_XS2 4
+#endif
+template <typename R, int PPT, int MODE>
+constexpr int min_blocks() {
+    return sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift ? ABP_BLOCKS_XS2 : 0;
+}
+
 // Steps [n, n_end) of every slot.  Folds happen after absolute multiples of
 // kBlockSteps steps; counter blocks are absolute multiples of 4.
-template <typename R, int PPT, int MODE = kModeEM, int UNROLL = kGroupUnroll>
+template <typename R, int PPT, int MODE = kModeEM, int UNROLL = kGroupUnroll, bool SHARED = true>
 __device__ __forceinline__ void advance(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, int64_t n,
                                         int64_t n_end) {
     while (n < n_end) {
         const int64_t blk_end = min(n_end, (n | (int64_t)(kBlockSteps - 1)) + 1);
         while (n < blk_end && (n & 3)) {
-            single_step<R, PPT, MODE>(k, K, S, n);
+            single_step<R, PPT, MODE, SHARED>(k, K, S, n);
             ++n;
         }
         if (n < blk_end) {
             const uint32_t m_end = (uint32_t)(blk_end >> 2);
             uint32_t m = (uint32_t)(n >> 2);
 #pragma unroll UNROLL
-            for (; m < m_end; ++m) group_step<R, PPT, MODE>(k, K, S, m);
+            for (; m < m_end; ++m) group_step<R, PPT, MODE, SHARED>(k, K, S, m);
             n = (int64_t)m << 2;
         }
         while (n < blk_end) {
-            single_step<R, PPT, MODE>(k, K, S, n);
+            single_step<R, PPT, MODE, SHARED>(k, K, S, n);
             ++n;
         }
         if ((blk_end & (kBlockSteps - 1)) == 0) {
@@ -562,6 +573,12 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
         PACKED ? packed_set(b, tile, min(lane_base + (int)threadIdx.x, count - 1)) : set_t;
     const Coef<R> k = load_coef<R>(sizeof(R) == 4 ? b.coef_f : b.coef_d, b.params, set, nz.dt);
 
+    // The trajectories of a thread share the head of their counter blocks as long as
+    // their global ids share the high word; a tile astride a multiple of 2^32 (one tile,
+    // for some traj_base) forms each trajectory's own.
+    auto id_hi = [&](int64_t i) { return (uint32_t)(((uint64_t)i + nz.traj_base) >> 32); };
+    const bool one_hi = PPT == 1 || MODE == kModeXorshift || id_hi(first) == id_hi(first + count - 1);
+
     Slots<R, PPT> S;
     int64_t idx[PPT];
     bool act[PPT];
@@ -616,7 +633,12 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
         if constexpr (WS) {
             if (warp_live) advance_ws<MODE == kModeHeun>(k, S, n, seg_end, *wc);
         } else {
-            if (warp_live) advance<R, PPT, MODE, UNROLL>(k, K, S, n, seg_end);
+            if (warp_live) {
+                if (one_hi)
+                    advance<R, PPT, MODE, UNROLL>(k, K, S, n, seg_end);
+                else
+                    advance<R, PPT, MODE, 1, false>(k, K, S, n, seg_end);
+            }
         }
         n = seg_end;
         if (hist && (h.snap_every > 0 ? (n % h.snap_every == 0) : (n == N))) {
@@ -674,7 +696,7 @@ __device__ __forceinline__ void zero_hist(uint32_t *sh, const Hist &h) {
 // each taking blockDim.x consecutive trajectories of it), every tile over the
 // window [g0, g1).
 template <typename R, int PPT, bool PACKED, int MODE>
-__global__ void ABP_INTEGRATE_BOUNDS integrate_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz,
+__global__ void __launch_bounds__(kThreads, (min_blocks<R, PPT, MODE>())) integrate_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz,
                                                      KeyParam kp, int64_t g0, int64_t g1) {
     extern __shared__ uint32_t sh[];
     if constexpr (!PACKED) zero_hist(sh, h);
@@ -827,7 +849,7 @@ __device__ __forceinline__ void store_release(int32_t *p, int v) {
 // bounded: past q.wait_limit_ns the block records status 1 and every block
 // leaves at its next check, without touching the item.
 template <typename R, int PPT, int MODE>
-__global__ void ABP_INTEGRATE_BOUNDS persistent_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp,
+__global__ void __launch_bounds__(kThreads, (min_blocks<R, PPT, MODE>())) persistent_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp,
                                                       Queue q, int64_t g0, int64_t g1, int64_t seg) {
     extern __shared__ uint32_t sh[];
     __shared__ int s_tile, s_round;
