@@ -496,11 +496,13 @@ struct TilePlan {
     std::vector<int64_t> set_first, tile_first;
     std::vector<int32_t> set_packed, set_tile_begin, tile_count, tile_set, set_order;
     std::vector<int32_t> slot_set;  // [packed tiles][kThreads]: the set of each slot's trajectory
-    int32_t n_single = 0, n_unpacked = 0, narrow = 0, sub_single = 1, sub_packed = 1;
+    int32_t n_single = 0, n_unpacked = 0, narrow = 0, sub_single = 1, sub_packed = 1, packed_ppt = 1, packed_threads = kThreads;
 };
 
+// can_pair: the packed-tile integrator may hold two trajectories per thread (FP32 state,
+// counter-based noise).
 bool plan_tiles(int32_t n_sets, const int64_t *n_traj, const int64_t *n_steps, int sched, int ppt, bool checkpoints,
-                int sm_count, TilePlan &p) {
+                int sm_count, TilePlan &p, bool can_pair = true) {
     const int64_t tile = (int64_t)kThreads * ppt;
     const bool can_pack = sched == 1 && !checkpoints;
     p.set_first.assign((size_t)n_sets + 1, 0);
@@ -582,6 +584,36 @@ bool plan_tiles(int32_t n_sets, const int64_t *n_traj, const int64_t *n_steps, i
         p.narrow = w;
         p.sub_single = (int32_t)((tile + w - 1) / w);
         p.sub_packed = kThreads / w;
+    }
+    // Packed tiles outside narrow launches.  Each of an SM's four schedulers holds whole
+    // warps, so time grows in steps of the fullest scheduler's load, counted in warps of
+    // one trajectory per thread: u1 = ceil(W / schedulers) with one trajectory per thread
+    // in narrow blocks, 2 ceil(tiles / SMs) in blocks of a whole tile, u2 = 2 ceil(W2 /
+    // schedulers) with two (W, W2: warps of 32, of 64 trajectories).  Measured on
+    // one-trajectory sets, 2,000 Euler-Maruyama steps: about 41 u1 + 30 us in blocks of 64
+    // threads (32: the same), 41.3 u + 23 in whole tiles, 38.1 u2 + 29 with two per thread
+    // (any block width); Heun 64 and 61 us per unit.  So two per thread where 0.93 u2 <= u1:
+    // 228 tiles 154 us (u1 = 3) against 178 (u2 = 4) and 189 (whole tiles, before), 256
+    // tiles 179 against 197 and 189, 460 tiles 322 against 334 and 354, 2,000 tiles 1,090
+    // against 1,139 and 1,172.  With xorshift noise two per thread is slower (256 tiles 198
+    // against 178 us), the FP64 state has no paired instructions: one.
+    p.packed_ppt = 1;
+    p.packed_threads = p.narrow ? p.narrow : kThreads;
+    if (p.narrow == 0 && n_tiles > p.n_single) {
+        int64_t w1 = 0, w2 = 0;
+        for (int32_t t = p.n_single; t < n_tiles; ++t) {
+            w1 += (p.tile_count[t] + 31) / 32;
+            w2 += (p.tile_count[t] + 63) / 64;
+        }
+        const int64_t sms = std::max(sm_count, 1);
+        const int64_t u1 = (w1 + 4 * sms - 1) / (4 * sms), u2 = 2 * ((w2 + 4 * sms - 1) / (4 * sms));
+        const int64_t u256 = 2 * ((n_tiles - p.n_single + sms - 1) / sms);
+        if (can_pair && 93 * u2 <= 100 * u1) {
+            p.packed_ppt = 2;
+            p.packed_threads = kThreads / 2;
+        } else if (u1 < u256) {
+            p.packed_threads = 64;
+        }
     }
     return true;
 }
@@ -698,7 +730,7 @@ abp_status configure_batch(abp_ctx *ctx, int sched, int ppt, int64_t spl) {
     {
         TilePlan plan;
         if (!plan_tiles(n_sets, ctx->n_traj.data(), ctx->n_steps.data(), ctx->sched, ctx->ppt, ctx->cfg.checkpoint_every > 0, ctx->sm_count,
-                        plan))
+                        plan, ctx->cfg.state_fp64 == 0 && ctx->cfg.noise == 0))
             return fail(ctx, ABP_EINVAL, "too many tiles");
         ctx->set_first.swap(plan.set_first);
         ctx->set_packed.swap(plan.set_packed);
@@ -714,6 +746,8 @@ abp_status configure_batch(abp_ctx *ctx, int sched, int ppt, int64_t spl) {
         ctx->narrow = plan.narrow;
         ctx->sub_single = plan.sub_single;
         ctx->sub_packed = plan.sub_packed;
+        ctx->packed_ppt = plan.packed_ppt;
+        ctx->packed_threads = plan.packed_threads;
     }
     const abp_config &c = ctx->cfg;
     const bool any_hist = c.hist_x_bins > 0 || c.hist_v_bins > 0;

@@ -86,6 +86,7 @@ struct abp_ctx {
     int32_t n_single = 0;  // tiles [n_single, n_tiles) are packed
     int32_t n_unpacked = 0;  // sets in one-set tiles
     int32_t narrow = 0, sub_single = 1, sub_packed = 1;  // narrow lockstep launch (small batches)
+    int32_t packed_ppt = 1, packed_threads = abp::kThreads;  // packed tiles: trajectories per thread, block width
 
     // device
     DevBuf d_params, d_steps, d_set_tile_begin, d_tile_first, d_tile_count, d_tile_set, d_set_first, d_set_order,
@@ -127,6 +128,8 @@ struct abp_ctx {
         b.narrow = narrow;
         b.sub_single = sub_single;
         b.sub_packed = sub_packed;
+        b.packed_ppt = packed_ppt;
+        b.packed_threads = packed_threads;
         b.params = (const abp_params *)d_params.p;
         b.set_steps = (const int64_t *)d_steps.p;
         b.set_tile_begin = (const int32_t *)d_set_tile_begin.p;

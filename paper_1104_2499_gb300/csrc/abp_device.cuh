@@ -347,28 +347,30 @@ __device__ __forceinline__ void heun_step_f32(const Coef<float> &k, float nrs, f
 
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 
-// The coefficients of Coef<float> that the paired step reads, duplicated into
-// both halves of a pair.
+// The coefficients of Coef<float> that the paired step reads, one per half of a pair.
 struct Coef2 {
     float2 A, nBd, Bd, Cq, Gd, F, K, A4, dtL, bm, Cm, hdtL;
 };
 
-__device__ __forceinline__ Coef2 make_coef2(const Coef<float> &k) {
+// The pair's coefficients: `a` in the first half, `b` in the second (the same set in
+// both, or each half its own set in packed tiles).
+__device__ __forceinline__ Coef2 make_coef2(const Coef<float> &a, const Coef<float> &b) {
     Coef2 c;
-    c.A = dup2(k.A);
-    c.nBd = dup2(-k.Bd);
-    c.Bd = dup2(k.Bd);
-    c.Cq = dup2(k.Cq);
-    c.Gd = dup2(k.Gd);
-    c.F = dup2(k.F);
-    c.K = dup2(k.K);
-    c.A4 = dup2(k.A4);
-    c.dtL = dup2(k.dtL);
-    c.bm = dup2(k.bm);
-    c.Cm = dup2(k.Cm);
-    c.hdtL = dup2(k.hdtL);
+    c.A = make_float2(a.A, b.A);
+    c.nBd = make_float2(-a.Bd, -b.Bd);
+    c.Bd = make_float2(a.Bd, b.Bd);
+    c.Cq = make_float2(a.Cq, b.Cq);
+    c.Gd = make_float2(a.Gd, b.Gd);
+    c.F = make_float2(a.F, b.F);
+    c.K = make_float2(a.K, b.K);
+    c.A4 = make_float2(a.A4, b.A4);
+    c.dtL = make_float2(a.dtL, b.dtL);
+    c.bm = make_float2(a.bm, b.bm);
+    c.Cm = make_float2(a.Cm, b.Cm);
+    c.hdtL = make_float2(a.hdtL, b.hdtL);
     return c;
 }
+__device__ __forceinline__ Coef2 make_coef2(const Coef<float> &k) { return make_coef2(k, k); }
 
 // box_muller_f32 of two word pairs (wa.x, wb.x) and (wa.y, wb.y), same
 // operations in the same order.

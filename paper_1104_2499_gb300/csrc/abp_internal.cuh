@@ -36,6 +36,9 @@ struct Batch {
     // threads (0: off), one trajectory per thread, sub_single blocks per one-set
     // tile and sub_packed per packed tile.  Tiles, and so every result, are the same.
     int32_t narrow, sub_single, sub_packed;
+    // Packed tiles of the lockstep integrator: trajectories per thread (1; 2: FP32 state
+    // only) and threads per block (a divisor of kThreads / packed_ppt, a multiple of 32).
+    int32_t packed_ppt = 1, packed_threads = kThreads;
     const abp_params *params;      // [n_sets]
     const int64_t *set_steps;      // [n_sets] steps to run
     const int32_t *set_tile_begin; // [n_sets + 1]

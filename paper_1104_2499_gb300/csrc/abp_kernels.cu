@@ -229,6 +229,13 @@ struct Pair {
     }
 };
 
+// The step coefficients of a thread's slots: one set for all of them, or (OWN) one set each.
+template <typename R, int PPT, bool OWN = false>
+struct Coefs {
+    Coef<R> k[OWN ? PPT : 1];
+    __device__ __forceinline__ const Coef<R> &of(int q) const { return k[OWN ? q : 0]; }
+};
+
 // Whether the FP32 slots of a thread are stepped in pairs.
 template <typename R, int PPT>
 constexpr bool kPaired = sizeof(R) == 4 && PPT % 2 == 0 && ABP_F32X2 && ABP_ANGLE_FFMA;
@@ -236,12 +243,12 @@ constexpr bool kPaired = sizeof(R) == 4 && PPT % 2 == 0 && ABP_F32X2 && ABP_ANGL
 // One Euler-Maruyama step of every slot at an arbitrary step index n (the
 // unaligned head / tail of a range): the counter block of n is generated for
 // this step alone.
-template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true>
-__device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, int64_t n) {
+template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true, bool OWN = false>
+__device__ __forceinline__ void single_step(const Coefs<R, PPT, OWN> &ks, const RoundKeys &K, Slots<R, PPT> &S, int64_t n) {
     if constexpr (MODE == kModeXorshift && kPaired<R, PPT>) {
-        const Coef2 k2 = make_coef2(k);
 #pragma unroll
         for (int p = 0; p < PPT; p += 2) {
+            const Coef2 k2 = make_coef2(ks.of(p), ks.of(p + 1));
             Pair<PPT> P(S, p);
             uint2 wa, wb;
             wa.x = xorshift128(S.xs[p]);
@@ -257,6 +264,7 @@ __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K
     } else if constexpr (MODE == kModeXorshift) {
 #pragma unroll
         for (int q = 0; q < PPT; ++q) {
+            const Coef<R> &k = ks.of(q);
             float nrs, cs, sn;
             const uint32_t wa = xorshift128(S.xs[q]);
             const uint32_t wb = xorshift128(S.xs[q]);
@@ -269,6 +277,7 @@ __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K
     const BlockHead head = block_head((uint32_t)(n >> 2), S.ss[0].hx);
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
+        const Coef<R> &k = ks.of(q);
         const uint4 w = SHARED ? step_block(head, S.ss[q], K) : step_block((uint32_t)(n >> 2), S.ss[q], K);
         if constexpr (sizeof(R) == 4) {
             float nrs, cs, sn;
@@ -286,11 +295,11 @@ __device__ __forceinline__ void single_step(const Coef<R> &k, const RoundKeys &K
 
 // Four steps 4m .. 4m+3 of every slot from one counter block each.  SHARED: the
 // slots' global ids have one high word, so one block head serves them all.
-template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true>
-__device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, uint32_t m) {
+template <typename R, int PPT, int MODE = kModeEM, bool SHARED = true, bool OWN = false>
+__device__ __forceinline__ void group_step(const Coefs<R, PPT, OWN> &ks, const RoundKeys &K, Slots<R, PPT> &S, uint32_t m) {
     if constexpr (MODE == kModeXorshift) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) single_step<R, PPT, MODE>(k, K, S, 0);
+        for (int i = 0; i < 4; ++i) single_step<R, PPT, MODE>(ks, K, S, 0);
         return;
     }
     constexpr bool HEUN = MODE == kModeHeun;
@@ -300,9 +309,9 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
     for (int q = 0; q < PPT; ++q) w[q] = SHARED ? step_block(head, S.ss[q], K) : step_block(m, S.ss[q], K);
     if constexpr (kPaired<R, PPT>) {
         // trajectories 2p and 2p + 1 in the two halves of FP32 register pairs
-        const Coef2 k2 = make_coef2(k);
 #pragma unroll
         for (int p = 0; p < PPT; p += 2) {
+            const Coef2 k2 = make_coef2(ks.of(p), ks.of(p + 1));
             Pair<PPT> P(S, p);
             float2 nr, cs, sn;
             box_muller_f32x2(make_uint2(w[p].x, w[p + 1].x), make_uint2(w[p].y, w[p + 1].y), k2.bm, nr, cs, sn);
@@ -316,20 +325,21 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
     } else if constexpr (sizeof(R) == 4) {
         float nr[PPT], cs[PPT], sn[PPT];
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) box_muller_f32(w[q].x, w[q].y, k.bm, nr[q], cs[q], sn[q]);
+        for (int q = 0; q < PPT; ++q) box_muller_f32(w[q].x, w[q].y, ks.of(q).bm, nr[q], cs[q], sn[q]);
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(k, nr[q], cs[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
+        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(ks.of(q), nr[q], cs[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(k, nr[q], sn[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
+        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(ks.of(q), nr[q], sn[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) box_muller_f32(w[q].z, w[q].w, k.bm, nr[q], cs[q], sn[q]);
+        for (int q = 0; q < PPT; ++q) box_muller_f32(w[q].z, w[q].w, ks.of(q).bm, nr[q], cs[q], sn[q]);
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(k, nr[q], cs[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
+        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(ks.of(q), nr[q], cs[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
 #pragma unroll
-        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(k, nr[q], sn[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
+        for (int q = 0; q < PPT; ++q) step_f32<HEUN>(ks.of(q), nr[q], sn[q], S.pb[q], S.yacc[q], S.v[q], S.e[q]);
     } else {
 #pragma unroll
         for (int q = 0; q < PPT; ++q) {
+            const Coef<R> &k = ks.of(q);
             double z0, z1, z2, z3;
             box_muller_f64(w[q].x, w[q].y, z0, z1);
             box_muller_f64(w[q].z, w[q].w, z2, z3);
@@ -364,9 +374,11 @@ __device__ __forceinline__ void group_step(const Coef<R> &k, const RoundKeys &K,
 #ifndef ABP_UNROLL_XS2
 #define ABP_UNROLL_XS2 8
 #endif
-template <typename R, int PPT, int MODE, bool QUEUE>
+template <typename R, int PPT, int MODE, bool QUEUE, bool PACKED = false>
 constexpr int group_unroll() {
-    if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeEM)
+    if constexpr (PACKED && PPT == 2)
+        return kGroupUnroll;  // coefficients of two sets: 4 blocks 350 us for 65,536 sets x 4,000 steps, 2 352, 8 351
+    else if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeEM)
         return QUEUE ? ABP_UNROLL_EM2_QUEUE : ABP_UNROLL_EM2;
     else if constexpr (sizeof(R) == 4 && PPT == 2 && MODE == kModeHeun)
         return ABP_UNROLL_HEUN2;
@@ -386,31 +398,31 @@ constexpr int group_unroll() {
 #ifndef ABP_BLOCKS_XS2
 #define ABP_BLOCKS_XS2 4
 #endif
-template <typename R, int PPT, int MODE>
+template <typename R, int PPT, int MODE, bool PACKED = false>
 constexpr int min_blocks() {
-    return sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift ? ABP_BLOCKS_XS2 : 0;
+    return !PACKED && sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift ? ABP_BLOCKS_XS2 : 0;
 }
 
 // Steps [n, n_end) of every slot.  Folds happen after absolute multiples of
 // kBlockSteps steps; counter blocks are absolute multiples of 4.
-template <typename R, int PPT, int MODE = kModeEM, int UNROLL = kGroupUnroll, bool SHARED = true>
-__device__ __forceinline__ void advance(const Coef<R> &k, const RoundKeys &K, Slots<R, PPT> &S, int64_t n,
+template <typename R, int PPT, int MODE = kModeEM, int UNROLL = kGroupUnroll, bool SHARED = true, bool OWN = false>
+__device__ __forceinline__ void advance(const Coefs<R, PPT, OWN> &ks, const RoundKeys &K, Slots<R, PPT> &S, int64_t n,
                                         int64_t n_end) {
     while (n < n_end) {
         const int64_t blk_end = min(n_end, (n | (int64_t)(kBlockSteps - 1)) + 1);
         while (n < blk_end && (n & 3)) {
-            single_step<R, PPT, MODE, SHARED>(k, K, S, n);
+            single_step<R, PPT, MODE, SHARED>(ks, K, S, n);
             ++n;
         }
         if (n < blk_end) {
             const uint32_t m_end = (uint32_t)(blk_end >> 2);
             uint32_t m = (uint32_t)(n >> 2);
 #pragma unroll UNROLL
-            for (; m < m_end; ++m) group_step<R, PPT, MODE, SHARED>(k, K, S, m);
+            for (; m < m_end; ++m) group_step<R, PPT, MODE, SHARED>(ks, K, S, m);
             n = (int64_t)m << 2;
         }
         while (n < blk_end) {
-            single_step<R, PPT, MODE, SHARED>(k, K, S, n);
+            single_step<R, PPT, MODE, SHARED>(ks, K, S, n);
             ++n;
         }
         if ((blk_end & (kBlockSteps - 1)) == 0) {
@@ -548,16 +560,18 @@ __device__ __forceinline__ void advance_ws(const Coef<float> &k, Slots<float, 1>
 // state), step it in registers, fill snapshot histograms and checkpoints, and
 // store it back.  Must be reached by every thread of the block; `sh` holds
 // zeros on entry (when histograms are on) and on exit.
-// PACKED: a packed tile (several sets of equal step count, PPT 1): each thread
+// PACKED: a packed tile (several sets of equal step count, PPT 1 or 2): each slot
 // takes the coefficients of its own trajectory's set, and histograms go to
-// global memory directly.
+// global memory directly.  The block takes trajectories [lane_base, lane_base +
+// PPT blockDim.x) of the tile.
 // WS: the consumer threads of a warp-specialised block (noise from the ring
 // of `wc`, histogram flushes on the consumers' own barrier).
 template <typename R, int PPT, bool PACKED = false, int MODE = kModeEM, int UNROLL = kGroupUnroll, bool WS = false>
 __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const Hist &h, const Ckpt &ck,
                                          const Noise &nz, const RoundKeys &K, uint32_t *sh, int tile, int64_t w0,
                                          int64_t w1, int lane_base = 0, WsCons *wc = nullptr) {
-    static_assert(!PACKED || PPT == 1, "packed tiles hold one trajectory per thread");
+    static_assert(!PACKED || PPT <= 2, "packed tiles hold one or two trajectories per thread");
+    constexpr bool OWN = PACKED && PPT > 1;  // the slots of a thread belong to different sets
     static_assert(!WS || (sizeof(R) == 4 && PPT == 1), "WS: FP32, one trajectory per thread");
     tile = (int)dchk(tile, b.n_tiles, b.dbg);
     const int64_t first = b.tile_first[tile];
@@ -569,9 +583,6 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
     if (n_begin >= n_end) return;  // uniform over the block
 
     const SV<R> s = view<R>(st);
-    const int set =
-        PACKED ? packed_set(b, tile, min(lane_base + (int)threadIdx.x, count - 1)) : set_t;
-    const Coef<R> k = load_coef<R>(sizeof(R) == 4 ? b.coef_f : b.coef_d, b.params, set, nz.dt);
 
     // The trajectories of a thread share the head of their counter blocks as long as
     // their global ids share the high word; a tile astride a multiple of 2^32 (one tile,
@@ -580,7 +591,9 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
     const bool one_hi = PPT == 1 || MODE == kModeXorshift || id_hi(first) == id_hi(first + count - 1);
 
     Slots<R, PPT> S;
+    Coefs<R, PPT, OWN> ks;
     int64_t idx[PPT];
+    int set[PACKED ? PPT : 1];
     bool act[PPT];
     // Thread t takes trajectories t, t + stride, ... of the tile.  A full tile has
     // stride kThreads; a partial one (the last tile of a set) ceil(count / PPT), so its
@@ -588,12 +601,19 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
     // idle (their issue slots go to the SM's other blocks) instead of every thread
     // carrying one real and PPT - 1 empty slots through the paired instructions.  A
     // trajectory's arithmetic does not depend on its thread or slot: same results.
-    const int stride = PPT > 1 ? (count + PPT - 1) / PPT : kThreads;
+    const int span = PACKED ? min(count - lane_base, PPT * (int)blockDim.x) : count;
+    const int stride = PPT > 1 ? (span + PPT - 1) / PPT : kThreads;
 #pragma unroll
     for (int q = 0; q < PPT; ++q) {
         const int li = lane_base + threadIdx.x + q * stride;
-        act[q] = (int)threadIdx.x < stride && li < count;
-        idx[q] = dchk(first + (act[q] ? li : count - 1), b.total_traj, b.dbg);
+        act[q] = (int)threadIdx.x < stride && li < (PPT > 1 ? lane_base + span : count);
+        const int slot = act[q] ? li : count - 1;
+        idx[q] = dchk(first + slot, b.total_traj, b.dbg);
+        if (PACKED || q == 0) {
+            set[PACKED ? q : 0] = PACKED ? packed_set(b, tile, slot) : set_t;
+            if (OWN || q == 0)
+                ks.k[OWN ? q : 0] = load_coef<R>(sizeof(R) == 4 ? b.coef_f : b.coef_d, b.params, set[PACKED ? q : 0], nz.dt);
+        }
         S.y[q] = __ldcg(&s.y[idx[q]]);
         S.yacc[q] = __ldcg(&s.yacc[idx[q]]);
         S.ylo[q] = __ldcg(&s.ylo[idx[q]]);
@@ -631,24 +651,26 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
         if (hist && h.snap_every > 0) seg_end = min(seg_end, (n / h.snap_every + 1) * h.snap_every);
         if (ck.every > 0) seg_end = min(seg_end, (n / ck.every + 1) * ck.every);
         if constexpr (WS) {
-            if (warp_live) advance_ws<MODE == kModeHeun>(k, S, n, seg_end, *wc);
+            if (warp_live) advance_ws<MODE == kModeHeun>(ks.of(0), S, n, seg_end, *wc);
         } else {
             if (warp_live) {
                 if (one_hi)
-                    advance<R, PPT, MODE, UNROLL>(k, K, S, n, seg_end);
+                    advance<R, PPT, MODE, UNROLL>(ks, K, S, n, seg_end);
                 else
-                    advance<R, PPT, MODE, 1, false>(k, K, S, n, seg_end);
+                    advance<R, PPT, MODE, 1, false>(ks, K, S, n, seg_end);
             }
         }
         n = seg_end;
         if (hist && (h.snap_every > 0 ? (n % h.snap_every == 0) : (n == N))) {
             const int64_t snap = dchk(h.snap_every > 0 ? n / h.snap_every - 1 : 0, h.n_snap, b.dbg);
             if constexpr (PACKED) {
-                if (act[0]) {
-                    const size_t row = (size_t)snap * b.n_sets + set;
-                    if (h.bx > 0) atomicAdd(&h.x[row * h.bx + bin_x<R>(S.y[0] + S.yacc[0], h.bx)], 1u);
+#pragma unroll
+                for (int q = 0; q < PPT; ++q) {
+                    if (!act[q]) continue;
+                    const size_t row = (size_t)snap * b.n_sets + set[q];
+                    if (h.bx > 0) atomicAdd(&h.x[row * h.bx + bin_x<R>(S.y[q] + S.yacc[q], h.bx)], 1u);
                     if (h.bv > 0)
-                        atomicAdd(&h.v[row * (h.bv + 2) + bin_v<R>(S.v[0], v_lo, v_hi, v_scale, h.bv)], 1u);
+                        atomicAdd(&h.v[row * (h.bv + 2) + bin_v<R>(S.v[q], v_lo, v_hi, v_scale, h.bv)], 1u);
                 }
             } else {
 #pragma unroll
@@ -657,7 +679,7 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
                     if (h.bx > 0) atomicAdd(&sh[bin_x<R>(S.y[q] + S.yacc[q], h.bx)], 1u);
                     if (h.bv > 0) atomicAdd(&sh[h.bx + bin_v<R>(S.v[q], v_lo, v_hi, v_scale, h.bv)], 1u);
                 }
-                flush_hist<WS>(sh, h, snap, set, b.n_sets, 32);
+                flush_hist<WS>(sh, h, snap, set[0], b.n_sets, 32);
             }
         }
         if (ck.every > 0 && n % ck.every == 0 && sizeof(R) == 4) {
@@ -692,19 +714,22 @@ __device__ __forceinline__ void zero_hist(uint32_t *sh, const Hist &h) {
     }
 }
 
-// Lockstep schedule: one block per tile (narrow launch: `sub` blocks per tile,
-// each taking blockDim.x consecutive trajectories of it), every tile over the
-// window [g0, g1).
+// Lockstep schedule: every tile over the window [g0, g1).  One-set tiles: one block per
+// tile, or in a narrow launch sub_single blocks, each taking blockDim.x consecutive
+// trajectories.  Packed tiles: blocks of any width w, each taking PPT w consecutive
+// trajectories.
 template <typename R, int PPT, bool PACKED, int MODE>
-__global__ void __launch_bounds__(kThreads, (min_blocks<R, PPT, MODE>())) integrate_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz,
-                                                     KeyParam kp, int64_t g0, int64_t g1) {
+__global__ void __launch_bounds__(PACKED ? kThreads / PPT : kThreads, (min_blocks<R, PPT, MODE, PACKED>()))
+    integrate_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp, int64_t g0, int64_t g1) {
     extern __shared__ uint32_t sh[];
     if constexpr (!PACKED) zero_hist(sh, h);
-    const int sub = b.narrow ? (PACKED ? b.sub_packed : b.sub_single) : 1;
+    const int per_block = (int)blockDim.x * (PACKED ? PPT : 1);
+    const int sub = PACKED ? kThreads / per_block : b.narrow ? b.sub_single : 1;
     const int tile = (PACKED ? b.n_single : 0) + (int)blockIdx.x / sub;
-    const int lane_base = ((int)blockIdx.x % sub) * (int)blockDim.x;
-    run_tile<R, PPT, PACKED, MODE, group_unroll<R, PPT, MODE, false>()>(b, st, h, ck, nz, kp.K, sh, tile, g0, g1,
-                                                                       lane_base);
+    const int lane_base = ((int)blockIdx.x % sub) * per_block;
+    if (PACKED && lane_base >= b.tile_count[tile]) return;  // past a short tile (packed tiles use no block barrier)
+    run_tile<R, PPT, PACKED, MODE, group_unroll<R, PPT, MODE, false, PACKED>()>(b, st, h, ck, nz, kp.K, sh, tile, g0, g1,
+                                                                               lane_base);
 }
 
 // Producer warp p of NP: the (nrs, trig) pairs of the launch's slots for the
@@ -1218,12 +1243,22 @@ cudaError_t launch_integrate_t(const Batch &b, const State &s, const Hist &h, co
         }
     }
     const int threads = b.narrow ? b.narrow : kThreads;
-    const int64_t sub_s = b.narrow ? b.sub_single : 1, sub_p = b.narrow ? b.sub_packed : 1;
+    const int64_t sub_s = b.narrow ? b.sub_single : 1;
+    const unsigned n_packed = (unsigned)(b.n_tiles - b.n_single);
     if (b.n_single > 0)
         kern<<<(unsigned)(b.n_single * sub_s), threads, smem, st>>>(b, s, h, c, nz, key_param(nz.k0, nz.k1), g0, g1);
-    if (b.n_tiles > b.n_single)  // packed tiles: one trajectory per thread, histograms in global memory
-        integrate_kernel<R, 1, true, MODE><<<(unsigned)((b.n_tiles - b.n_single) * sub_p), threads, 0, st>>>(
-            b, s, h, c, nz, key_param(nz.k0, nz.k1), g0, g1);
+    if (n_packed > 0) {  // histograms in global memory
+        const int w = b.packed_threads;
+        const unsigned grid = n_packed * (unsigned)(kThreads / (w * b.packed_ppt));
+        const KeyParam kp = key_param(nz.k0, nz.k1);
+        bool paired = false;
+        if constexpr (sizeof(R) == 4 && MODE != kModeXorshift) {
+            paired = b.packed_ppt == 2;
+            if (paired) integrate_kernel<R, 2, true, MODE><<<grid, w, 0, st>>>(b, s, h, c, nz, kp, g0, g1);
+        }
+        if (!paired && b.packed_ppt != 1) return cudaErrorInvalidValue;
+        if (!paired) integrate_kernel<R, 1, true, MODE><<<grid, w, 0, st>>>(b, s, h, c, nz, kp, g0, g1);
+    }
     return cudaGetLastError();
 }
 
