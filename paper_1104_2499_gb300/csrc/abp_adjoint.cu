@@ -69,15 +69,35 @@ constexpr int kL1Threads = 128;
 constexpr int kSub = ABP_ADJ_SUB;  // steps per register-resident sub-chunk (a multiple of 4)
 static_assert(kSub % 4 == 0 && (kBlockSteps % kSub) == 0, "sub-chunks hold whole Philox blocks");
 
+// Sub-chunks lie on absolute multiples of kSub steps (not on offsets from the segment's
+// start, where a checkpoint interval that is no multiple of kSub sent every chunk of most
+// segments down the one-step-at-a-time path: 262,144 trajectories x 4,000 steps, forward
+// and backward, K = 500 5.93 -> 3.98 ms, K = 333 7.60 -> 4.21 ms), so that a whole chunk holds whole
+// Philox blocks and no position fold falls inside it whatever the segment's start: the
+// segment [s0, s1) has chunks c0 = s0 / kSub .. (s1 - 1) / kSub, the first and the last
+// of them possibly partial (when checkpoint_every or the run's length is not a multiple
+// of kSub).
+struct SegChunks {
+    int64_t s0, s1, c0;  // the segment's steps and its first chunk
+    int n;               // its chunks
+    __device__ __forceinline__ SegChunks(int64_t a, int64_t b) : s0(a), s1(b), c0(a / kSub), n((int)((b + kSub - 1) / kSub - a / kSub)) {}
+    __device__ __forceinline__ int64_t begin(int j) const { return j == 0 ? s0 : (c0 + j) * kSub; }
+    __device__ __forceinline__ int64_t end(int j) const { return j == n - 1 ? s1 : (c0 + j + 1) * kSub; }
+    __device__ __forceinline__ bool whole(int j) const { return end(j) - begin(j) == kSub; }
+    // chunks [first_whole, last_whole) are whole
+    __device__ __forceinline__ int first_whole() const { return s0 % kSub ? 1 : 0; }
+    __device__ __forceinline__ int last_whole() const { return max(s1 % kSub ? n - 1 : n, first_whole()); }
+};
+
 struct AdjArgs {
     Batch b;
     Ckpt ck;
     Noise nz;
     RoundKeys K;        // Philox round keys of the seed (constant bank)
     float4 *sub;        // [n_sub][total_traj] sub-checkpoints (scratch)
-    int64_t n_sub;      // sub-checkpoint slots per segment
+    int64_t n_sub;      // sub-checkpoint slots per segment (sub_slots)
     uint4 *words;       // [block][n_blk][2][threads] noise hand-off of the segment (scratch), WORDS kernels only
-    int64_t n_blk;      // Philox blocks per segment (checkpoint_every / 4)
+    int64_t n_blk;      // Philox blocks per segment (kSub / 4 per sub-checkpoint slot)
     const double *w;    // [n_sets] dJ/dmean_v, NULL = 1
     double *partials;   // [n_tiles][6]
 };
@@ -127,8 +147,8 @@ __device__ __forceinline__ void block_noise(const Coef<float> &k, const StepStre
     tr[3] = s;
 }
 
-// The same noise one step at a time, for segments that do not start on a
-// multiple of 8 steps (one Philox block kept for its four steps).
+// The same noise one step at a time, for partial chunks (one Philox block kept for its
+// four steps).
 struct NoiseCursor {
     uint32_t m;
     bool valid;
@@ -212,25 +232,22 @@ __device__ __forceinline__ void block_sum6(double (&a)[6], double (*red)[6]) {
 }
 
 // Level 1 of segment [s0, s1) of one trajectory: re-run from its checkpoint
-// (y, yacc, v, e) = c0, leaving the state at s0, s0 + kSub, ... in the
-// sub-checkpoint scratch.  Segments that start on a multiple of kSub steps run
-// in whole kSub-step chunks whose noise comes one Philox block per four steps
-// (the forward's own path); others step one at a time.
+// (y, yacc, v, e) = c0, leaving the state at the start of each chunk in the
+// sub-checkpoint scratch.  Whole chunks take their noise one Philox block per four
+// steps (the forward's own path); partial ones step one at a time.
 __device__ __forceinline__ void level1_segment(const AdjArgs &a, const Coef<float> &k, const StepStream &ss,
                                                int64_t idx, int64_t s0, int64_t s1, float4 c0) {
     const int64_t T = a.b.total_traj;
+    const SegChunks seg(s0, s1);
     float y = c0.x, yacc = c0.y, v = c0.z, e = c0.w;
     float pb = phase_base(y);
-    const int n_chunks = (int)((s1 - s0 + kSub - 1) / kSub);
-    const bool aligned = (s0 & (kSub - 1)) == 0;
     NoiseCursor nc;
     nc.valid = false;
     nc.m = 0;
-    for (int j = 0; j < n_chunks; ++j) {
-        const int64_t n0 = s0 + (int64_t)j * kSub;
+    for (int j = 0; j < seg.n; ++j) {
+        const int64_t n0 = seg.begin(j);
         a.sub[(size_t)dchk(j, a.n_sub, a.b.dbg) * T + idx] = make_float4(y, yacc, v, e);
-        const int len = (int)(s1 - n0 < kSub ? s1 - n0 : kSub);
-        if (aligned && len == kSub) {
+        if (seg.whole(j)) {
 #pragma unroll
             for (int b2 = 0; b2 < kSub / 4; ++b2) {
                 float nrs[4], tr[4];
@@ -240,6 +257,7 @@ __device__ __forceinline__ void level1_segment(const AdjArgs &a, const Coef<floa
             }
             if (((n0 + kSub) & (kBlockSteps - 1)) == 0) fold(y, yacc, pb);
         } else {
+            const int len = (int)(seg.end(j) - n0);
             for (int i = 0; i < len; ++i) {
                 float nrs, tr;
                 nc.at(k, ss, a.K, n0 + i, nrs, tr);
@@ -250,7 +268,7 @@ __device__ __forceinline__ void level1_segment(const AdjArgs &a, const Coef<floa
 }
 
 // level1_segment for two trajectories (idx0, idx1) of one thread: whole
-// aligned chunks step the pair with paired FP32 instructions (same operations
+// chunks step the pair with paired FP32 instructions (same operations
 // as em_step_f32 / box_muller_f32 on each half, so the sub-checkpoints are the
 // scalar ones bit for bit); other chunks step each trajectory on its own.
 // store1: whether the second trajectory is real (else it duplicates the first
@@ -290,105 +308,71 @@ __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<flo
                                                 const int64_t (&idx)[2], bool store1, int64_t s0, int64_t s1,
                                                 float4 c0, float4 c1) {
     const int64_t T = a.b.total_traj;
+    const SegChunks seg(s0, s1);
     uint4 *const wp = WORDS ? a.words + (size_t)blockIdx.x * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x : nullptr;
-    float y[2] = {c0.x, c1.x}, yacc[2] = {c0.y, c1.y}, v[2] = {c0.z, c1.z}, e[2] = {c0.w, c1.w};
-    float pb[2] = {phase_base(y[0]), phase_base(y[1])};
-    const int n_chunks = (int)((s1 - s0 + kSub - 1) / kSub);
-    const bool aligned = (s0 & (kSub - 1)) == 0;
+    float y[2] = {c0.x, c1.x};
+    float2 Y = make_float2(c0.y, c1.y), V = make_float2(c0.z, c1.z), E = make_float2(c0.w, c1.w);
+    float2 PB = make_float2(phase_base(y[0]), phase_base(y[1]));
     const Coef2 k2 = make_coef2(k);
-    NoiseCursor nc[2];
-    nc[0].valid = nc[1].valid = false;
-    nc[0].m = nc[1].m = 0;
-    int j = 0;
-#if ABP_ADJ_L1_GROUP > 1
-    // aligned whole chunks in groups of ABP_ADJ_L1_GROUP: one loop iteration per group
-    if (aligned) {
-        const int full = (int)((s1 - s0) / kSub);
-        float2 Y = make_float2(yacc[0], yacc[1]), V = make_float2(v[0], v[1]), E = make_float2(e[0], e[1]);
-        float2 PB = make_float2(pb[0], pb[1]);
-        for (; j + ABP_ADJ_L1_GROUP <= full; j += ABP_ADJ_L1_GROUP) {
-#pragma unroll
-            for (int c = 0; c < ABP_ADJ_L1_GROUP; ++c) {
-                const int jc = j + c;
-                const int64_t n0 = s0 + (int64_t)jc * kSub;
-                const size_t js = (size_t)dchk(jc, a.n_sub, a.b.dbg);
-                a.sub[js * T + idx[0]] = make_float4(y[0], Y.x, V.x, E.x);
-                if (store1) a.sub[js * T + idx[1]] = make_float4(y[1], Y.y, V.y, E.y);
-#pragma unroll
-                for (int b2 = 0; b2 < kSub / 4; ++b2) {
-                    const uint32_t m = (uint32_t)(n0 >> 2) + b2;
-                    uint4 w0, w1;
-                    pair_blocks(m, ss, a.K, w0, w1);
-                    float2 nrA, nrB, cs, sn;
-                    box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nrA, cs, sn);
-                    em_step_f32x2(k2, nrA, cs, PB, Y, V, E);
-                    em_step_f32x2(k2, nrA, sn, PB, Y, V, E);
-                    box_muller_f32x2(make_uint2(w0.z, w1.z), make_uint2(w0.w, w1.w), k2.bm, nrB, cs, sn);
-                    em_step_f32x2(k2, nrB, cs, PB, Y, V, E);
-                    em_step_f32x2(k2, nrB, sn, PB, Y, V, E);
-                    store_words<WORDS>(a, wp, 2 * (int64_t)jc + b2, w0, w1, nrA, nrB);
-                }
-                if (((n0 + kSub) & (kBlockSteps - 1)) == 0) {
-                    yacc[0] = Y.x;
-                    yacc[1] = Y.y;
-                    fold(y[0], yacc[0], pb[0]);
-                    fold(y[1], yacc[1], pb[1]);
-                    Y = make_float2(yacc[0], yacc[1]);
-                    PB = make_float2(pb[0], pb[1]);
-                }
-            }
-        }
-        yacc[0] = Y.x;
-        yacc[1] = Y.y;
-        v[0] = V.x;
-        v[1] = V.y;
-        e[0] = E.x;
-        e[1] = E.y;
-    }
-#endif
-    for (; j < n_chunks; ++j) {
-        const int64_t n0 = s0 + (int64_t)j * kSub;
+    auto store = [&](int j) {
         const size_t js = (size_t)dchk(j, a.n_sub, a.b.dbg);
-        a.sub[js * T + idx[0]] = make_float4(y[0], yacc[0], v[0], e[0]);
-        if (store1) a.sub[js * T + idx[1]] = make_float4(y[1], yacc[1], v[1], e[1]);
-        const int len = (int)(s1 - n0 < kSub ? s1 - n0 : kSub);
-        if (aligned && len == kSub) {
-            float2 Y = make_float2(yacc[0], yacc[1]), V = make_float2(v[0], v[1]), E = make_float2(e[0], e[1]);
-            const float2 PB = make_float2(pb[0], pb[1]);
+        a.sub[js * T + idx[0]] = make_float4(y[0], Y.x, V.x, E.x);
+        if (store1) a.sub[js * T + idx[1]] = make_float4(y[1], Y.y, V.y, E.y);
+    };
+    auto whole_chunk = [&](int j) {
+        const int64_t n0 = (seg.c0 + j) * kSub;
+        store(j);
 #pragma unroll
-            for (int b2 = 0; b2 < kSub / 4; ++b2) {
-                const uint32_t m = (uint32_t)(n0 >> 2) + b2;
-                uint4 w0, w1;
-                pair_blocks(m, ss, a.K, w0, w1);
-                float2 nrA, nrB, cs, sn;
-                box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nrA, cs, sn);
-                em_step_f32x2(k2, nrA, cs, PB, Y, V, E);
-                em_step_f32x2(k2, nrA, sn, PB, Y, V, E);
-                box_muller_f32x2(make_uint2(w0.z, w1.z), make_uint2(w0.w, w1.w), k2.bm, nrB, cs, sn);
-                em_step_f32x2(k2, nrB, cs, PB, Y, V, E);
-                em_step_f32x2(k2, nrB, sn, PB, Y, V, E);
-                store_words<WORDS>(a, wp, 2 * (int64_t)j + b2, w0, w1, nrA, nrB);
-            }
-            yacc[0] = Y.x;
-            yacc[1] = Y.y;
-            v[0] = V.x;
-            v[1] = V.y;
-            e[0] = E.x;
-            e[1] = E.y;
-            if (((n0 + kSub) & (kBlockSteps - 1)) == 0) {
-                fold(y[0], yacc[0], pb[0]);
-                fold(y[1], yacc[1], pb[1]);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < 2; ++q)
-                for (int i = 0; i < len; ++i) {
-                    float nrs, tr;
-                    nc[q].at(k, ss[q], a.K, n0 + i, nrs, tr);
-                    fwd(k, nrs, tr, n0 + i, y[q], yacc[q], pb[q], v[q], e[q]);
-                }
+        for (int b2 = 0; b2 < kSub / 4; ++b2) {
+            uint4 w0, w1;
+            pair_blocks((uint32_t)(n0 >> 2) + b2, ss, a.K, w0, w1);
+            float2 nrA, nrB, cs, sn;
+            box_muller_f32x2(make_uint2(w0.x, w1.x), make_uint2(w0.y, w1.y), k2.bm, nrA, cs, sn);
+            em_step_f32x2(k2, nrA, cs, PB, Y, V, E);
+            em_step_f32x2(k2, nrA, sn, PB, Y, V, E);
+            box_muller_f32x2(make_uint2(w0.z, w1.z), make_uint2(w0.w, w1.w), k2.bm, nrB, cs, sn);
+            em_step_f32x2(k2, nrB, cs, PB, Y, V, E);
+            em_step_f32x2(k2, nrB, sn, PB, Y, V, E);
+            store_words<WORDS>(a, wp, (kSub / 4) * (int64_t)j + b2, w0, w1, nrA, nrB);
         }
+        if (((n0 + kSub) & (kBlockSteps - 1)) == 0) {
+            fold(y[0], Y.x, PB.x);
+            fold(y[1], Y.y, PB.y);
+        }
+    };
+    auto partial_chunk = [&](int j) {  // each trajectory on its own
+        store(j);
+        const int64_t n0 = seg.begin(j), n1 = seg.end(j);
+#pragma unroll 1
+        for (int q = 0; q < 2; ++q) {
+            const StepStream sq = q ? ss[1] : ss[0];
+            float yq = q ? y[1] : y[0], ya = q ? Y.y : Y.x, v = q ? V.y : V.x, e = q ? E.y : E.x, pb = q ? PB.y : PB.x;
+            NoiseCursor nc;
+            nc.valid = false;
+            nc.m = 0;
+            for (int64_t n = n0; n < n1; ++n) {
+                float nrs, tr;
+                nc.at(k, sq, a.K, n, nrs, tr);
+                fwd(k, nrs, tr, n, yq, ya, pb, v, e);
+            }
+            if (q) {
+                y[1] = yq, Y.y = ya, V.y = v, E.y = e, PB.y = pb;
+            } else {
+                y[0] = yq, Y.x = ya, V.x = v, E.x = e, PB.x = pb;
+            }
+        }
+    };
+    const int j1 = seg.last_whole();
+    int j = 0;
+    if (j < seg.first_whole()) partial_chunk(j++);
+    // whole chunks in groups of ABP_ADJ_L1_GROUP: one loop iteration per group
+    for (; j + ABP_ADJ_L1_GROUP <= j1; j += ABP_ADJ_L1_GROUP) {
+#pragma unroll
+        for (int c = 0; c < ABP_ADJ_L1_GROUP; ++c) whole_chunk(j + c);
     }
+#pragma unroll 1
+    for (; j < j1; ++j) whole_chunk(j);
+    if (j < seg.n) partial_chunk(j);
 }
 
 // Level 2 and the reverse sweep of segment [s0, s1): its kSub-step chunks in
@@ -399,22 +383,21 @@ __device__ __forceinline__ void reverse_chunks(const AdjArgs &a, const Coef<floa
                                                float dtf, int64_t idx, int64_t s0, int64_t s1, float &lx, float &lv,
                                                float &le, float (&acc)[6]) {
     const int64_t T = a.b.total_traj;
-    const int n_chunks = (int)((s1 - s0 + kSub - 1) / kSub);
-    const bool aligned = (s0 & (kSub - 1)) == 0;
+    const SegChunks seg(s0, s1);
     NoiseCursor nc;
     nc.valid = false;
     nc.m = 0;
-    float4 c_next = a.sub[(size_t)dchk(n_chunks - 1, a.n_sub, a.b.dbg) * T + idx];
-    for (int j = n_chunks - 1; j >= 0; --j) {
-        const int64_t n0 = s0 + (int64_t)j * kSub;
-        const int len = (int)(s1 - n0 < kSub ? s1 - n0 : kSub);
+    float4 c_next = a.sub[(size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg) * T + idx];
+    for (int j = seg.n - 1; j >= 0; --j) {
+        const int64_t n0 = seg.begin(j);
+        const int len = (int)(seg.end(j) - n0);
         const float4 cj = c_next;
         if (j > 0) c_next = a.sub[(size_t)dchk(j - 1, a.n_sub, a.b.dbg) * T + idx];
         float y = cj.x, yacc = cj.y, v = cj.z, e = cj.w;
         float pb = phase_base(y);
         float ys[kSub], vs[kSub], es[kSub], szs[kSub];  // ys: the force phase of each step
-        if (aligned && len == kSub) {
-            // no fold falls inside an aligned chunk (folds come after multiples of kBlockSteps)
+        if (len == kSub) {
+            // no fold falls inside a whole chunk (folds come after multiples of kBlockSteps)
 #pragma unroll
             for (int b2 = 0; b2 < kSub / 4; ++b2) {
                 float nrs[4], tr[4];
@@ -502,7 +485,7 @@ __device__ __forceinline__ void reverse_step_x2(const RevCoef2 &c, float2 ph, fl
 }
 
 // reverse_chunks for two trajectories of one thread (idx[0], idx[1]): whole
-// aligned chunks run the level-2 re-run and the reverse sweep on FP32 pairs;
+// chunks run the level-2 re-run and the reverse sweep on FP32 pairs;
 // other chunks run each trajectory on its own with the scalar functions.
 // Shared-memory stage of the hand-off: [kStages][kSub / 4 blocks][2 trajectories][thread].
 typedef uint4 WordStage[kSub / 4][2][kRevPairThreads];
@@ -513,9 +496,8 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
                                                 float2 &lx, float2 &lv, float2 &le, float2 (&acc)[6],
                                                 WordStage *stage) {
     const int64_t T = a.b.total_traj;
-    const int n_chunks = (int)((s1 - s0 + kSub - 1) / kSub);
-    const bool aligned = (s0 & (kSub - 1)) == 0;
-    const int full = aligned ? (int)((s1 - s0) / kSub) : 0;  // chunks 0 .. full - 1 are whole
+    const SegChunks seg(s0, s1);
+    const int j0w = seg.first_whole(), j1w = seg.last_whole();  // chunks [j0w, j1w) are whole
     const Coef2 k2 = make_coef2(k);
     const RevCoef2 rc = make_rev_coef2(k, kx, dtf);
     // WORDS: copy whole chunk jj's blocks into stage[jj % kStages]; one commit group per
@@ -523,11 +505,11 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     const uint4 *const wr =
         WORDS ? a.words + (size_t)blockIdx.x * (size_t)a.n_blk * (2 * kRevPairThreads) + threadIdx.x : nullptr;
     auto fetch = [&](int jj) {
-        if (jj >= 0 && jj < full) {
+        if (jj >= j0w && jj < j1w) {
             WordStage &st = stage[jj % kStages];
 #pragma unroll
             for (int b2 = 0; b2 < kSub / 4; ++b2) {
-                const int64_t r = dchk(2 * (int64_t)jj + b2, a.n_blk, a.b.dbg) * (2 * kRevPairThreads);
+                const int64_t r = dchk((kSub / 4) * (int64_t)jj + b2, a.n_blk, a.b.dbg) * (2 * kRevPairThreads);
                 cp_async16(&st[b2][0][threadIdx.x], wr + r);
                 cp_async16(&st[b2][1][threadIdx.x], wr + r + kRevPairThreads);
             }
@@ -536,12 +518,10 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     };
     if (WORDS)
 #pragma unroll
-        for (int i = 0; i < kStages - 1; ++i) fetch(n_chunks - 1 - i);
-    const size_t jl = (size_t)dchk(n_chunks - 1, a.n_sub, a.b.dbg);
+        for (int i = 0; i < kStages - 1; ++i) fetch(seg.n - 1 - i);
+    const size_t jl = (size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg);
     float4 n0c = a.sub[jl * T + idx[0]], n1c = a.sub[jl * T + idx[1]];
-    for (int j = n_chunks - 1; j >= 0; --j) {
-        const int64_t n0 = s0 + (int64_t)j * kSub;
-        const int len = (int)(s1 - n0 < kSub ? s1 - n0 : kSub);
+    for (int j = seg.n - 1; j >= 0; --j) {
         const float4 c0 = n0c, c1 = n1c;
         if (j > 0) {
             const size_t jp = (size_t)dchk(j - 1, a.n_sub, a.b.dbg);
@@ -552,7 +532,8 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
             fetch(j - (kStages - 1));
             cp_async_wait<kStages - 1>();  // this thread's copies of chunk j have landed
         }
-        if (aligned && len == kSub) {
+        if (j >= j0w && j < j1w) {
+            const int64_t n0 = (seg.c0 + j) * kSub;
             float2 Y = make_float2(c0.y, c1.y), V = make_float2(c0.z, c1.z), E = make_float2(c0.w, c1.w);
             const float2 PB = make_float2(phase_base(c0.x), phase_base(c1.x));
             float2 ys[kSub], vs[kSub], es[kSub], szs[kSub];
@@ -596,7 +577,9 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
 #pragma unroll
             for (int i = kSub - 1; i >= 0; --i) reverse_step_x2(rc, ys[i], vs[i], es[i], szs[i], lx, lv, le, acc);
         } else {
-            // scalar path, one trajectory after the other
+            // a partial chunk: scalar path, one trajectory after the other
+            const int64_t n0 = seg.begin(j);
+            const int len = (int)(seg.end(j) - n0);
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const float4 cq = q ? c1 : c0;
@@ -879,6 +862,10 @@ struct AdjLayout {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Sub-checkpoint slots of a segment of K steps: the chunks it can touch (SegChunks), one
+// more than K / kSub rounded up when segments start anywhere on the chunk grid.
+int64_t sub_slots(int64_t K) { return (K + kSub - 1) / kSub + (K % kSub ? 1 : 0); }
+
 // Kernel blocks per tile of the paired level-1 and reverse kernels (tiles hold up
 // to kThreads * ppt trajectories, a block two per thread).
 int pair_blocks_per_tile(const abp_ctx *ctx, int threads) {
@@ -889,7 +876,7 @@ int pair_blocks_per_tile(const abp_ctx *ctx, int threads) {
 AdjLayout adj_layout(const abp_ctx *ctx, bool words) {
     AdjLayout L;
     const int64_t T = ctx->total_traj, Kc = ctx->cfg.checkpoint_every;
-    const int64_t n_sub = (Kc + kSub - 1) / kSub;
+    const int64_t n_sub = sub_slots(Kc);
     L.sub1 = sizeof(float4) * (size_t)n_sub * (size_t)T;
     L.sub = 2 * align256(L.sub1);  // two buffers, alternating by segment
     L.part = sizeof(double) * 6 * (size_t)std::max(ctx->n_tiles, 1);
@@ -898,7 +885,7 @@ AdjLayout adj_layout(const abp_ctx *ctx, bool words) {
     L.lam = sizeof(float4) * (size_t)std::max<int64_t>(T, 1);
     L.g = sizeof(double) * 6 * (size_t)std::max<int64_t>(T, 1);
     const size_t blocks = (size_t)ctx->n_tiles * (size_t)pair_blocks_per_tile(ctx, kL1Threads);
-    L.words1 = words ? sizeof(uint4) * blocks * (size_t)(Kc / 4) * 2 * kL1Threads : 0;
+    L.words1 = words ? sizeof(uint4) * blocks * (size_t)(n_sub * (kSub / 4)) * 2 * kL1Threads : 0;
     L.words = 2 * align256(L.words1);
     L.off_part = align256(L.sub);
     L.off_grad = L.off_part + align256(L.part);
@@ -911,13 +898,11 @@ AdjLayout adj_layout(const abp_ctx *ctx, bool words) {
 }
 
 // Whether abp_backward hands the Philox blocks from level 1 to the reverse sweep:
-// the paired kernels, segments of whole sub-chunks, and both buffers within the
-// budget -- ABP_ADJ_HANDOFF_BYTES if set (0: never), else half the free device
+// the paired kernels and both buffers within the budget -- ABP_ADJ_HANDOFF_BYTES if set (0: never), else half the free device
 // memory not already held by the scratch.
 bool use_handoff(const abp_ctx *ctx) {
     // both kernels must map blocks and threads to trajectories alike
     if (!ABP_ADJ_L1_PAIRS || !ABP_ADJ_REV_PAIRS || kL1Threads != kRevPairThreads) return false;
-    if (ctx->cfg.checkpoint_every % kSub != 0) return false;
     const size_t bytes = adj_layout(ctx, true).words;
     const char *env = getenv("ABP_ADJ_HANDOFF_BYTES");
     if (env && *env) return (double)bytes <= strtod(env, nullptr);
@@ -952,7 +937,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     if (ctx->g < ctx->max_steps) return set_err(ctx, ABP_ESTATE, "abp_backward before the integration completed");
     if (!ctx->ckpt_complete)
         return set_err(ctx, ABP_ESTATE, "abp_backward after abp_load: the checkpoints do not cover the run from step 0");
-    const int64_t n_sub = (ctx->cfg.checkpoint_every + kSub - 1) / kSub;
+    const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
     bool words = use_handoff(ctx);
     AdjLayout L = adj_layout(ctx, words);
     DevBuf &sc = ctx->d_adj;
@@ -1007,7 +992,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         a.sub = sub[0];
         a.n_sub = n_sub;
         a.words = nullptr;
-        a.n_blk = ctx->cfg.checkpoint_every / 4;
+        a.n_blk = n_sub * (kSub / 4);
         a.w = w;
         a.partials = partials;
         for (int r = 0; r < 10; ++r) {
@@ -1104,7 +1089,7 @@ extern "C" abp_status abp_backward_traj(abp_ctx *ctx, double *dvbar) {
     const int64_t T = ctx->total_traj;
     if (T == 0 || ctx->n_tiles == 0) return ABP_OK;
     // the per-trajectory sums of the last backward call: the same scratch layout as there
-    const int64_t n_sub = (ctx->cfg.checkpoint_every + kSub - 1) / kSub;
+    const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
     const AdjLayout L = adj_layout(ctx, false);  // the hand-off buffers come after the sums
     char *base = (char *)ctx->d_adj.p;
     SegView sv;
