@@ -98,6 +98,7 @@ struct AdjArgs {
     int64_t n_sub;      // sub-checkpoint slots per segment (sub_slots)
     uint4 *words;       // [block][n_blk][2][threads] noise hand-off of the segment (scratch), WORDS kernels only
     int64_t n_blk;      // Philox blocks per segment (kSub / 4 per sub-checkpoint slot)
+    int tile0;          // first tile of the launch (its group of tiles)
     const double *w;    // [n_sets] dJ/dmean_v, NULL = 1
     double *partials;   // [n_tiles][6]
 };
@@ -306,10 +307,10 @@ __device__ __forceinline__ void pair_blocks(uint32_t m, const StepStream (&ss)[2
 template <bool WORDS>
 __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<float> &k, const StepStream (&ss)[2],
                                                 const int64_t (&idx)[2], bool store1, int64_t s0, int64_t s1,
-                                                float4 c0, float4 c1) {
+                                                float4 c0, float4 c1, int block) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
-    uint4 *const wp = WORDS ? a.words + (size_t)blockIdx.x * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x : nullptr;
+    uint4 *const wp = WORDS ? a.words + (size_t)block * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x : nullptr;
     float y[2] = {c0.x, c1.x};
     float2 Y = make_float2(c0.y, c1.y), V = make_float2(c0.z, c1.z), E = make_float2(c0.w, c1.w);
     float2 PB = make_float2(phase_base(y[0]), phase_base(y[1]));
@@ -494,7 +495,7 @@ template <bool WORDS>
 __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<float> &k, const StepStream (&ss)[2],
                                                 float kx, float dtf, const int64_t (&idx)[2], int64_t s0, int64_t s1,
                                                 float2 &lx, float2 &lv, float2 &le, float2 (&acc)[6],
-                                                WordStage *stage) {
+                                                WordStage *stage, int block) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
     const int j0w = seg.first_whole(), j1w = seg.last_whole();  // chunks [j0w, j1w) are whole
@@ -503,7 +504,7 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     // WORDS: copy whole chunk jj's blocks into stage[jj % kStages]; one commit group per
     // call, empty for chunks that are not whole, so that groups and chunks stay in step
     const uint4 *const wr =
-        WORDS ? a.words + (size_t)blockIdx.x * (size_t)a.n_blk * (2 * kRevPairThreads) + threadIdx.x : nullptr;
+        WORDS ? a.words + (size_t)block * (size_t)a.n_blk * (2 * kRevPairThreads) + threadIdx.x : nullptr;
     auto fetch = [&](int jj) {
         if (jj >= j0w && jj < j1w) {
             WordStage &st = stage[jj % kStages];
@@ -626,14 +627,16 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     }
 }
 
-// One launch per segment index and level, segments in reverse order: level 1
-// (a plain forward re-run, light on registers) for segment `seg` of every
-// trajectory, then level 2 and the reverse sweep (register-heavy) for the same
-// segment.  The level-1 launch of segment seg - 1 runs on a second stream
-// while the reverse sweep of segment seg runs, into the other of two
-// sub-checkpoint buffers.  Between launches each trajectory keeps its adjoint
+// One launch per segment index, level and group of tiles, segments in reverse
+// order: level 1 (a plain forward re-run, light on registers) for segment `seg`
+// of the group's trajectories, then level 2 and the reverse sweep
+// (register-heavy) for the same segment.  The level-1 launch of segment seg - 1
+// runs on a second stream while the reverse sweep of segment seg runs, into the
+// other of two sub-checkpoint buffers.  Between launches each trajectory keeps its adjoint
 // state lambda = (x, v, e) and its six gradient sums in global memory.
 // Trajectories of sets shorter than seg K skip.
+constexpr int kAdjGroups = abp_ctx::kAdjGroups;
+
 struct SegView {
     float4 *lam;  // [total_traj] (lambda_x, lambda_v, lambda_e, -)
     double *G;    // [6][total_traj] gradient sums
@@ -643,7 +646,7 @@ struct SegView {
 // its trajectories [j blockDim, (j + 1) blockDim): one trajectory per thread.
 __global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, int64_t seg, int sub) {
     const Batch &b = a.b;
-    const int tile = (int)blockIdx.x / sub;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
@@ -662,7 +665,7 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, i
 template <bool WORDS>
 __global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs a, int64_t seg, int sub) {
     const Batch &b = a.b;
-    const int tile = (int)blockIdx.x / sub;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * 2 * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
@@ -679,14 +682,14 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs
                               step_stream((uint64_t)idx[1] + a.nz.traj_base, a.K)};
     const int64_t slot = dchk(seg, a.ck.n_slots, b.dbg);
     level1_segment2<WORDS>(a, k, ss, idx, second, s0, s1, a.ck.ck[(size_t)slot * T + idx[0]],
-                           a.ck.ck[(size_t)slot * T + idx[1]]);
+                           a.ck.ck[(size_t)slot * T + idx[1]], a.tile0 * sub + (int)blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kRevThreads, ABP_ADJ_MIN_BLOCKS) adjoint_reverse_kernel(AdjArgs a, SegView sv,
                                                                                           int64_t seg, int sub,
                                                                                           int64_t window) {
     const Batch &b = a.b;
-    const int tile = (int)blockIdx.x / sub;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
@@ -718,7 +721,7 @@ __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) 
                                                                                int sub, int64_t window) {
     __shared__ WordStage stage[WORDS ? kStages : 1];
     const Batch &b = a.b;
-    const int tile = (int)blockIdx.x / sub;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * 2 * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
@@ -742,7 +745,8 @@ __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) 
     float2 acc[6];
 #pragma unroll
     for (int q = 0; q < 6; ++q) acc[q] = make_float2(0.0f, 0.0f);
-    reverse_chunks2<WORDS>(a, k, ss, kx, dtf, idx, s0, s1, lx, lv, le, acc, stage);
+    reverse_chunks2<WORDS>(a, k, ss, kx, dtf, idx, s0, s1, lx, lv, le, acc, stage,
+                           a.tile0 * sub + (int)blockIdx.x);
     sv.lam[idx[0]] = make_float4(lx.x, lv.x, le.x, 0.0f);
 #pragma unroll
     for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[0]] += (double)acc[q].x;
@@ -992,6 +996,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         a.sub = sub[0];
         a.n_sub = n_sub;
         a.words = nullptr;
+        a.tile0 = 0;
         a.n_blk = n_sub * (kSub / 4);
         a.w = w;
         a.partials = partials;
@@ -1002,61 +1007,101 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         e = cudaMemsetAsync(sv.lam, 0, lam_bytes, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(sv.G, 0, g_bytes, s);
         if (e != cudaSuccess) return set_err(ctx, ABP_ECUDA, "abp_backward: clear", e);
-        if (!ctx->aux) {
-            e = cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking);
-            for (int i = 0; e == cudaSuccess && i < 5; ++i)
+        const int64_t Kc = ctx->cfg.checkpoint_every;
+        const int64_t n_seg = (ctx->max_steps + Kc - 1) / Kc;
+        // blocks per tile: tiles hold up to kThreads * ppt trajectories
+        const int cap = kThreads * std::max(ctx->ppt, 1);
+        const int sub1 = ABP_ADJ_L1_PAIRS ? pair_blocks_per_tile(ctx, kL1Threads) : (cap + kL1Threads - 1) / kL1Threads;
+        const int sub2 = ABP_ADJ_REV_PAIRS ? pair_blocks_per_tile(ctx, kRevPairThreads)
+                                           : (cap + kRevThreads - 1) / kRevThreads;
+        // The tiles in two halves, each with its own pair of streams: a trajectory's sweep
+        // depends on no other's, so while one half's launch of a segment drains (its last
+        // blocks fill the SMs partly, and its next launch waits for them) the other half's
+        // blocks take the free SMs.  Backward of one set, K = 1,000, against one group:
+        // 262,144 trajectories 2.67 -> 2.48 ps per particle-step, 175,104 2.91 -> 2.56,
+        // 131,072 3.09 -> 2.71, 1,048,576 2.40 -> 2.38 (three, four and six groups: within 2%
+        // of two).  A batch with fewer blocks than SMs runs in one group: it leaves SMs
+        // free anyway, and each launch costs host time.
+        const int n_grp = ctx->n_tiles >= 2 && (int64_t)ctx->n_tiles * sub2 >= ctx->sm_count ? kAdjGroups : 1;
+        if (!ctx->adj_stream[0]) {
+            for (int i = 0; e == cudaSuccess && i < 2 * kAdjGroups - 1; ++i)
+                e = cudaStreamCreateWithFlags(&ctx->adj_stream[i], cudaStreamNonBlocking);
+            for (int i = 0; e == cudaSuccess && i < abp_ctx::kAdjEvents; ++i)
                 e = cudaEventCreateWithFlags(&ctx->adj_ev[i], cudaEventDisableTiming);
             if (e != cudaSuccess) {
                 ctx->release_streams();
                 return set_err(ctx, ABP_ECUDA, "abp_backward: stream set-up", e);
             }
         }
-        cudaStream_t s2 = ctx->aux;
-        cudaEvent_t *l1_done = ctx->adj_ev, *rev_done = ctx->adj_ev + 2, start = ctx->adj_ev[4];
-        const int64_t Kc = ctx->cfg.checkpoint_every;
-        const int64_t n_seg = (ctx->max_steps + Kc - 1) / Kc;
+        struct Group {
+            cudaStream_t rev, l1;
+            cudaEvent_t *l1_done, *rev_done;  // [2] by segment parity
+            int t0, t1;
+        } grp[kAdjGroups];
+        for (int g = 0; g < n_grp; ++g) {
+            grp[g].rev = g == 0 ? s : ctx->adj_stream[2 * g];
+            grp[g].l1 = ctx->adj_stream[g == 0 ? 0 : 2 * g - 1];
+            grp[g].l1_done = ctx->adj_ev + 2 + 4 * g;
+            grp[g].rev_done = ctx->adj_ev + 4 + 4 * g;
+            grp[g].t0 = (int)((int64_t)ctx->n_tiles * g / n_grp);
+            grp[g].t1 = (int)((int64_t)ctx->n_tiles * (g + 1) / n_grp);
+        }
+        const cudaEvent_t start = ctx->adj_ev[0], end = ctx->adj_ev[1];
+        auto wait = [&](cudaStream_t st, cudaEvent_t ev) {
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ev, 0);
+        };
+        auto record = [&](cudaEvent_t ev, cudaStream_t st) {
+            if (e == cudaSuccess) e = cudaEventRecord(ev, st);
+        };
         // level 1 of segment j writes buffer j % 2; it may start once the reverse
         // sweep of segment j + 2, the last reader of that buffer, has finished
-        e = cudaEventRecord(start, s);  // the checkpoints of the forward are complete
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, start, 0);
-        // blocks per tile: tiles hold up to kThreads * ppt trajectories
-        const int cap = kThreads * std::max(ctx->ppt, 1);
-        const int sub1 = ABP_ADJ_L1_PAIRS ? pair_blocks_per_tile(ctx, kL1Threads) : (cap + kL1Threads - 1) / kL1Threads;
-        const int sub2 = ABP_ADJ_REV_PAIRS ? pair_blocks_per_tile(ctx, kRevPairThreads)
-                                           : (cap + kRevThreads - 1) / kRevThreads;
-        auto level1 = [&](int64_t j) {
+        auto level1 = [&](const Group &g, int64_t j) {
             AdjArgs aj = a;
             aj.sub = sub[j & 1];
-            const unsigned g1 = (unsigned)((int64_t)ctx->n_tiles * sub1);
+            aj.tile0 = g.t0;
+            const unsigned g1 = (unsigned)((int64_t)(g.t1 - g.t0) * sub1);
             if (words) {
                 aj.words = wbuf[j & 1];
-                adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, s2>>>(aj, j, sub1);
+                adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
             } else if (ABP_ADJ_L1_PAIRS)
-                adjoint_level1_pair_kernel<false><<<g1, kL1Threads, 0, s2>>>(aj, j, sub1);
+                adjoint_level1_pair_kernel<false><<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
             else
-                adjoint_level1_kernel<<<(unsigned)((int64_t)ctx->n_tiles * sub1), kL1Threads, 0, s2>>>(aj, j, sub1);
-            return cudaEventRecord(l1_done[j & 1], s2);
+                adjoint_level1_kernel<<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
+            record(g.l1_done[j & 1], g.l1);
         };
-        if (e == cudaSuccess && n_seg > 0) e = level1(n_seg - 1);
-        for (int64_t seg = n_seg - 1; e == cudaSuccess && seg >= 0; --seg) {
-            if (seg > 0) {
-                if (seg + 1 < n_seg) e = cudaStreamWaitEvent(s2, rev_done[(seg + 1) & 1], 0);
-                if (e == cudaSuccess) e = level1(seg - 1);
-            }
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(s, l1_done[seg & 1], 0);
+        auto reverse = [&](const Group &g, int64_t j) {
+            wait(g.rev, g.l1_done[j & 1]);
             AdjArgs as = a;
-            as.sub = sub[seg & 1];
-            const unsigned g2 = (unsigned)((int64_t)ctx->n_tiles * sub2);
+            as.sub = sub[j & 1];
+            as.tile0 = g.t0;
+            const unsigned g2 = (unsigned)((int64_t)(g.t1 - g.t0) * sub2);
             if (words) {
-                as.words = wbuf[seg & 1];
-                adjoint_reverse_pair_kernel<true><<<g2, kRevPairThreads, 0, s>>>(as, sv, seg, sub2, window);
+                as.words = wbuf[j & 1];
+                adjoint_reverse_pair_kernel<true><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j, sub2, window);
             } else if (ABP_ADJ_REV_PAIRS)
-                adjoint_reverse_pair_kernel<false><<<g2, kRevPairThreads, 0, s>>>(as, sv, seg, sub2, window);
+                adjoint_reverse_pair_kernel<false><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j, sub2, window);
             else
-                adjoint_reverse_kernel<<<(unsigned)((int64_t)ctx->n_tiles * sub2), kRevThreads, 0, s>>>(as, sv, seg,
-                                                                                                       sub2, window);
-            if (e == cudaSuccess) e = cudaEventRecord(rev_done[seg & 1], s);
+                adjoint_reverse_kernel<<<g2, kRevThreads, 0, g.rev>>>(as, sv, j, sub2, window);
+            record(g.rev_done[j & 1], g.rev);
             ctx->launches += 2;
+        };
+        record(start, s);  // the checkpoints of the forward and the cleared sums are complete
+        for (int g = 0; g < n_grp; ++g) {
+            wait(grp[g].l1, start);
+            if (g > 0) wait(grp[g].rev, start);
+            if (n_seg > 0) level1(grp[g], n_seg - 1);
+        }
+        for (int64_t seg = n_seg - 1; e == cudaSuccess && seg >= 0; --seg)
+            for (int g = 0; g < n_grp; ++g) {
+                if (seg > 0) {
+                    if (seg + 1 < n_seg) wait(grp[g].l1, grp[g].rev_done[(seg + 1) & 1]);
+                    level1(grp[g], seg - 1);
+                }
+                reverse(grp[g], seg);
+            }
+        for (int g = 1; g < n_grp; ++g) {  // also after an error: the caller's stream then follows all launches
+            cudaEventRecord(end, grp[g].rev);
+            cudaStreamWaitEvent(s, end, 0);
         }
         if (e != cudaSuccess) return set_err(ctx, ABP_ECUDA, "abp_backward: launch", e);
         adjoint_final_kernel<<<ctx->n_tiles, kThreads, 0, s>>>(a, sv);
@@ -1102,6 +1147,7 @@ extern "C" abp_status abp_backward_traj(abp_ctx *ctx, double *dvbar) {
     a.sub = nullptr;
     a.n_sub = n_sub;
     a.words = nullptr;
+    a.tile0 = 0;
     a.n_blk = 0;
     a.w = nullptr;
     a.partials = nullptr;

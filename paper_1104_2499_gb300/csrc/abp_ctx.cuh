@@ -101,8 +101,12 @@ struct abp_ctx {
     DevBuf d_hx, d_hv, d_ckpt, d_partials, d_moments, d_status;
     DevBuf d_queue, d_round, d_perm;  // work queue: head + done[n_tiles]; round starts; tile order
     DevBuf d_adj;  // adjoint scratch
-    cudaStream_t aux = nullptr;  // second stream of abp_backward (level-1 re-runs beside the reverse sweep)
-    cudaEvent_t adj_ev[5] = {};  // its ordering events
+    // abp_backward: the tiles in up to kAdjGroups groups, each with a stream for its level-1
+    // re-runs and one for its reverse sweeps (the first group's sweeps run on `stream`),
+    // and the ordering events: start, end, and two per stream and group.
+    static constexpr int kAdjGroups = 2, kAdjEvents = 2 + 4 * kAdjGroups;
+    cudaStream_t adj_stream[2 * kAdjGroups - 1] = {};
+    cudaEvent_t adj_ev[kAdjEvents] = {};
 
     // Live results (abp_live): snapshot k is copied to the caller's page-locked
     // buffers on live_stream once the main stream has passed step (k + 1) S.
@@ -207,7 +211,7 @@ struct abp_ctx {
     void release_streams() {
         if (live_stream) cudaStreamSynchronize(live_stream);
         for (cudaEvent_t *arr : {adj_ev + 0, live_done + 0, live_copied + 0}) {
-            const int n = arr == adj_ev ? 5 : kLiveRing;
+            const int n = arr == adj_ev ? kAdjEvents : kLiveRing;
             for (int i = 0; i < n; ++i)
                 if (arr[i]) {
                     cudaEventDestroy(arr[i]);
@@ -218,10 +222,11 @@ struct abp_ctx {
             cudaStreamDestroy(live_stream);
             live_stream = nullptr;
         }
-        if (aux) {
-            cudaStreamDestroy(aux);
-            aux = nullptr;
-        }
+        for (cudaStream_t &st : adj_stream)
+            if (st) {
+                cudaStreamDestroy(st);
+                st = nullptr;
+            }
     }
     void release_all() {
         if (live_stream) cudaStreamSynchronize(live_stream);
