@@ -450,8 +450,12 @@ __device__ __forceinline__ void advance(const Coefs<R, PPT, OWN> &ks, const Roun
 // each stored by one lane after a warp barrier with release semantics and read
 // with acquire semantics.  The consumer checks once per slot and only when its
 // last reading is used up; a check at a slot boundary costs it the drain of its
-// dependent chain, so slots are long: with 16-step slots the checks took about
-// 29 of 59 cycles per step, with 64-step slots about 4 of 34.
+// dependent chain, so slots are long and the check reads all producers' counters at
+// once: with 16-step slots the checks took about 29 of 59 cycles per step, with
+// 64-step slots about 4 of 34, with the counters read together 2 of 32 (4,096
+// trajectories x 10^4 steps 166 -> 157 us).  The chain alone takes 27.  Tried on top:
+// the slot handed back eight steps late, the next slot's counters read in mid-slot,
+// four or six slots, 16-byte reads of two steps: within 2% either way.
 // Every wait is bounded: past the wait limit the thread records status 1 and
 // stops waiting, so the launch runs to its end and the host reports the timeout.
 constexpr int kWsSlotSteps = 64;
@@ -516,6 +520,14 @@ struct WsCons {
     bool failed;
 };
 
+// The slots that every producer the consumer waits on has written: each lane reads
+// one producer's counter, so that the reads take one shared-memory latency together
+// instead of one each.
+__device__ __forceinline__ int32_t ws_filled(const WsCons &c) {
+    const int lane = threadIdx.x & 31;
+    return (int32_t)__reduce_min_sync(0xffffffffu, (uint32_t)ld_acquire_cta(&c.r.filled[lane < c.np ? lane : 0]));
+}
+
 // advance() with the noise taken from the ring (FP32, one trajectory per
 // thread; the producers drew it from the counter-based stream or from the
 // trajectory's xorshift generator).
@@ -528,8 +540,12 @@ __device__ __forceinline__ void advance_ws(const Coef<float> &k, Slots<float, 1>
         const int64_t a = n / SS;
         const int32_t kf = (int32_t)(a - c.a0);
         if (kf >= c.ready) {
-            int32_t rd = ws_wait(&c.r.filled[0], kf + 1, c.r, c.failed);
-            for (int p = 1; p < c.np; ++p) rd = min(rd, ws_wait(&c.r.filled[p], kf + 1, c.r, c.failed));
+            int32_t rd = ws_filled(c);
+            if (rd <= kf) {
+                for (int p = 0; p < c.np; ++p) ws_wait(&c.r.filled[p], kf + 1, c.r, c.failed);
+                c.failed = __any_sync(0xffffffffu, c.failed);  // the warp stops waiting as one
+                rd = kf + 1;
+            }
             c.ready = c.failed ? INT32_MAX : rd;
         }
         const float2 *ring = c.r.buf + (size_t)(kf % kWsSlots) * SS * 32 + lane;
@@ -804,6 +820,9 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
                 out[i * 32] = make_float2(nr, cs);
             }
         } else {
+            // two counter blocks at a time: a producer with its scheduler to itself is bound by
+            // the latency of a block's chain
+#pragma unroll 2
             for (int j = p; j < SS / 4; j += NP) {
                 const uint4 wv = step_block((uint32_t)(a * (SS / 4) + j), ss, K);
                 float nr, cs, sn;
