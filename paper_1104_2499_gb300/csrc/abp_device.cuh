@@ -277,14 +277,14 @@ __device__ __forceinline__ float phase_base(float y) {
 }
 __device__ __forceinline__ float phase_arg(float pb, float yacc) { return fmaf(yacc, kTwoPiF, pb); }
 
-// One Euler-Maruyama step; every right-hand side uses the step-n values.
-// `sz` is sigma * z_n.
+// One Euler-Maruyama step with the normal z_n; every right-hand side uses the step-n
+// values.
 template <typename R>
-__device__ __forceinline__ void em_step(const Coef<R> &k, R sz, R y, R &yacc, R &v, R &e) {
+__device__ __forceinline__ void em_step(const Coef<R> &k, R z, R y, R &yacc, R &v, R &e) {
     const R cphi = cos_phase(y + yacc);
     const R t1 = fma(-k.Bd, v * v, k.A);
     const R hv = fma(k.Bd, e, k.Gd);
-    const R a1 = sz + k.F;
+    const R a1 = fma(k.sigma, z, k.F);
     const R a2 = fma(hv, v, a1);
     const R P = fma(k.A4, cphi, k.K);
     const R dv = fma(P, cphi, a2);

@@ -288,7 +288,7 @@ __device__ __forceinline__ void single_step(const Coefs<R, PPT, OWN> &ks, const 
             step_f32<MODE == kModeHeun>(k, nrs, (j & 1) ? sn : cs, S.pb[q], S.yacc[q], S.v[q], S.e[q]);
         } else {
             const double z = normal_from_block_f64(w, j);
-            em_step<double>(k, k.sigma * z, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step<double>(k, z, S.y[q], S.yacc[q], S.v[q], S.e[q]);
         }
     }
 }
@@ -343,10 +343,10 @@ __device__ __forceinline__ void group_step(const Coefs<R, PPT, OWN> &ks, const R
             double z0, z1, z2, z3;
             box_muller_f64(w[q].x, w[q].y, z0, z1);
             box_muller_f64(w[q].z, w[q].w, z2, z3);
-            em_step<double>(k, k.sigma * z0, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, k.sigma * z1, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, k.sigma * z2, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, k.sigma * z3, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step<double>(k, z0, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step<double>(k, z1, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step<double>(k, z2, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step<double>(k, z3, S.y[q], S.yacc[q], S.v[q], S.e[q]);
         }
     }
 }
@@ -476,8 +476,18 @@ constexpr int kWsProducers = 3;
 #define ABP_WS_WIDEST 64
 #endif
 
+// One step's noise in the ring: (nrs, trig) of the FP32 state, the normal z of the FP64 state.
+template <typename R>
+struct WsNoise {
+    using T = float2;
+};
+template <>
+struct WsNoise<double> {
+    using T = double;
+};
+
 struct WsRing {
-    float2 *buf;        // [kWsSlots][kWsSlotSteps][32] (nrs, trig) per lane and step
+    void *buf;          // [kWsSlots][kWsSlotSteps][32] WsNoise per lane and step (8 bytes each)
     int32_t *filled;    // [NP]: slots of the launch written by producer warp p
     int32_t *consumed;  // slots of the launch the consumer warp has finished
     int32_t *status;    // 1 once a wait gave up
@@ -528,14 +538,20 @@ __device__ __forceinline__ int32_t ws_filled(const WsCons &c) {
     return (int32_t)__reduce_min_sync(0xffffffffu, (uint32_t)ld_acquire_cta(&c.r.filled[lane < c.np ? lane : 0]));
 }
 
-// advance() with the noise taken from the ring (FP32, one trajectory per
-// thread; the producers drew it from the counter-based stream or from the
-// trajectory's xorshift generator).
-template <bool HEUN>
-__device__ __forceinline__ void advance_ws(const Coef<float> &k, Slots<float, 1> &S, int64_t n, int64_t n_end,
-                                           WsCons &c) {
+// advance() with the noise taken from the ring (one trajectory per thread; the
+// producers drew it from the counter-based stream or from the trajectory's
+// xorshift generator).
+template <typename R, bool HEUN>
+__device__ __forceinline__ void advance_ws(const Coef<R> &k, Slots<R, 1> &S, int64_t n, int64_t n_end, WsCons &c) {
+    using T = typename WsNoise<R>::T;
     constexpr int SS = kWsSlotSteps;
     const int lane = threadIdx.x & 31;
+    auto step = [&](T t) {
+        if constexpr (sizeof(R) == 4)
+            step_f32<HEUN>(k, t.x, t.y, S.pb[0], S.yacc[0], S.v[0], S.e[0]);
+        else
+            em_step<double>(k, t, S.y[0], S.yacc[0], S.v[0], S.e[0]);
+    };
     while (n < n_end) {
         const int64_t a = n / SS;
         const int32_t kf = (int32_t)(a - c.a0);
@@ -548,24 +564,20 @@ __device__ __forceinline__ void advance_ws(const Coef<float> &k, Slots<float, 1>
             }
             c.ready = c.failed ? INT32_MAX : rd;
         }
-        const float2 *ring = c.r.buf + (size_t)(kf % kWsSlots) * SS * 32 + lane;
+        const T *ring = (const T *)c.r.buf + (size_t)(kf % kWsSlots) * SS * 32 + lane;
         const int64_t a_end = min(n_end, (a + 1) * SS);
         if (n == a * SS && a_end == (a + 1) * SS) {
-#pragma unroll
-            for (int i = 0; i < SS; ++i) {
-                const float2 t = ring[i * 32];
-                step_f32<HEUN>(k, t.x, t.y, S.pb[0], S.yacc[0], S.v[0], S.e[0]);
-            }
+            // an FP32 slot's body is unrolled whole; an FP64 step is some hundred instructions
+            constexpr int U = sizeof(R) == 4 ? SS : 2;
+#pragma unroll U
+            for (int i = 0; i < SS; ++i) step(ring[i * 32]);
         } else {
-            for (; n < a_end; ++n) {
-                const float2 t = ring[(int)(n - a * SS) * 32];
-                step_f32<HEUN>(k, t.x, t.y, S.pb[0], S.yacc[0], S.v[0], S.e[0]);
-            }
+            for (; n < a_end; ++n) step(ring[(int)(n - a * SS) * 32]);
         }
         n = a_end;
         if ((n & (kBlockSteps - 1)) == 0) {  // the slot's last step: fold, and hand the slot back
-            fold_position<float>(S.y[0], S.yacc[0], S.ylo[0], S.cell[0]);
-            S.pb[0] = phase_base(S.y[0]);
+            fold_position<R>(S.y[0], S.yacc[0], S.ylo[0], S.cell[0]);
+            if constexpr (sizeof(R) == 4) S.pb[0] = phase_base(S.y[0]);
             ws_publish(c.r.consumed, kf + 1);
         }
     }
@@ -588,7 +600,7 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
                                          int64_t w1, int lane_base = 0, WsCons *wc = nullptr) {
     static_assert(!PACKED || PPT <= 2, "packed tiles hold one or two trajectories per thread");
     constexpr bool OWN = PACKED && PPT > 1;  // the slots of a thread belong to different sets
-    static_assert(!WS || (sizeof(R) == 4 && PPT == 1), "WS: FP32, one trajectory per thread");
+    static_assert(!WS || PPT == 1, "WS: one trajectory per thread");
     tile = (int)dchk(tile, b.n_tiles, b.dbg);
     const int64_t first = b.tile_first[tile];
     const int count = b.tile_count[tile];
@@ -667,7 +679,7 @@ __device__ __forceinline__ void run_tile(const Batch &b, const State &st, const 
         if (hist && h.snap_every > 0) seg_end = min(seg_end, (n / h.snap_every + 1) * h.snap_every);
         if (ck.every > 0) seg_end = min(seg_end, (n / ck.every + 1) * ck.every);
         if constexpr (WS) {
-            if (warp_live) advance_ws<MODE == kModeHeun>(ks.of(0), S, n, seg_end, *wc);
+            if (warp_live) advance_ws<R, MODE == kModeHeun>(ks.of(0), S, n, seg_end, *wc);
         } else {
             if (warp_live) {
                 if (one_hi)
@@ -748,14 +760,14 @@ __global__ void __launch_bounds__(PACKED ? kThreads / PPT : kThreads, (min_block
                                                                                lane_base);
 }
 
-// Producer warp p of NP: the (nrs, trig) pairs of the launch's slots for the
+// Producer warp p of NP: the noise (WsNoise) of the launch's slots for the
 // 32 trajectories of the consumer warp (lane by lane), in slot order, a slot
 // rewritten only after the consumer handed it back.  The values are those
 // single_step / group_step compute: same counter blocks (or, with xorshift
 // noise, the same words of the trajectory's generator, which the first
 // producer loads, advances over the launch's steps and stores back), same
 // Box-Muller, same coefficient.
-template <bool PACKED, int MODE, int NP>
+template <typename R, bool PACKED, int MODE, int NP>
 __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, const Noise &nz, const RoundKeys &K,
                                            const WsRing &r, int tile, int64_t w0, int64_t w1, int lane_base, int p) {
     constexpr int SS = kWsSlotSteps;
@@ -773,7 +785,7 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
     if (!__any_sync(0xffffffffu, act)) return;  // the consumer warp does not step either
     if (tile == r.hold_tile) return;            // test hook: the consumer's waits run out
     const int set = PACKED ? packed_set(b, tile, min(li, count - 1)) : set_t;
-    const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, nz.dt);
+    const Coef<R> k = load_coef<R>(sizeof(R) == 4 ? b.coef_f : b.coef_d, b.params, set, nz.dt);
     const StepStream ss = step_stream((uint64_t)idx + nz.traj_base, K);
     const int64_t a0 = n_begin / SS, a1 = (n_end - 1) / SS;
     bool failed = false;
@@ -792,7 +804,7 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
             const int32_t c = ws_wait(r.consumed, kf + 1 - kWsSlots, r, failed);
             room = failed ? INT32_MAX : c + kWsSlots;
         }
-        float2 *out = r.buf + (size_t)(kf % kWsSlots) * SS * 32 + lane;
+        auto *out = (typename WsNoise<R>::T *)r.buf + (size_t)(kf % kWsSlots) * SS * 32 + lane;
         if constexpr (MODE == kModeXorshift) {
             // the generator advances only over the launch's own steps (two words and the
             // Box-Muller cosine per step, as single_step draws them); a whole chunk of 16
@@ -819,6 +831,15 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
                 box_muller_f32(wa, wb, k.bm, nr, cs, sn);
                 out[i * 32] = make_float2(nr, cs);
             }
+        } else if constexpr (sizeof(R) == 8) {
+            for (int j = p; j < SS / 4; j += NP) {
+                const uint4 wv = step_block((uint32_t)(a * (SS / 4) + j), ss, K);
+                double z[4];
+                box_muller_f64(wv.x, wv.y, z[0], z[1]);
+                box_muller_f64(wv.z, wv.w, z[2], z[3]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) out[(4 * j + i) * 32] = z[i];
+            }
         } else {
             // two counter blocks at a time: a producer with its scheduler to itself is bound by
             // the latency of a block's chain
@@ -841,12 +862,12 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
     }
 }
 
-// Warp-specialised narrow lockstep launch (FP32, any scheme and noise): blocks
+// Warp-specialised narrow lockstep launch (any state type, scheme and noise): blocks
 // of 32 (1 + NP) threads over the 32 trajectories a narrow block of 32 threads
 // takes (sub blocks per tile); warp 0 steps them (run_tile), warps 1..NP
 // produce their noise.  Dynamic shared memory: the histogram bins (one-set
 // tiles), then the ring at the next 16-byte boundary.
-template <bool PACKED, int MODE, int NP>
+template <typename R, bool PACKED, int MODE, int NP>
 __global__ void __launch_bounds__(32 * (1 + NP)) ws_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz,
                                                           KeyParam kp, int64_t g0, int64_t g1, WaitCtl wait) {
     extern __shared__ uint32_t sh[];
@@ -856,7 +877,7 @@ __global__ void __launch_bounds__(32 * (1 + NP)) ws_kernel(Batch b, State st, Hi
     if constexpr (!PACKED) zero_hist(sh, h);
     __syncthreads();
     const int nb = PACKED ? 0 : h.bx + (h.bv > 0 ? h.bv + 2 : 0);
-    float2 *ring = (float2 *)(sh + ((nb + 3) & ~3));
+    void *ring = sh + ((nb + 3) & ~3);
     if (smem_addr(ring) & 15) {  // uniform; never expected (dynamic shared memory is 16-byte aligned)
         if (threadIdx.x == 0) atomicCAS(wait.status, 0, 2);
         return;
@@ -868,9 +889,9 @@ __global__ void __launch_bounds__(32 * (1 + NP)) ws_kernel(Batch b, State st, Hi
     const int warp = (int)threadIdx.x >> 5;
     if (warp == 0) {
         WsCons c{r, MODE == kModeXorshift ? 1 : NP, 0, 0, false};
-        run_tile<float, 1, PACKED, MODE, kGroupUnroll, true>(b, st, h, ck, nz, kp.K, sh, tile, g0, g1, lane_base, &c);
+        run_tile<R, 1, PACKED, MODE, kGroupUnroll, true>(b, st, h, ck, nz, kp.K, sh, tile, g0, g1, lane_base, &c);
     } else {
-        ws_produce<PACKED, MODE, NP>(b, st, nz, kp.K, r, tile, g0, g1, lane_base, warp - 1);
+        ws_produce<R, PACKED, MODE, NP>(b, st, nz, kp.K, r, tile, g0, g1, lane_base, warp - 1);
     }
 }
 
@@ -1183,30 +1204,30 @@ cudaError_t launch_persistent_t(const Batch &b, const State &s, const Hist &h, c
 
 // Raise the kernel's dynamic shared-memory limit to `smem` (the ring alone is
 // 48 KB: with the static counters a block is past the default limit).
-template <bool PACKED, int MODE>
+template <typename R, bool PACKED, int MODE>
 cudaError_t ws_smem_limit(size_t smem) {
-    return cudaFuncSetAttribute(ws_kernel<PACKED, MODE, kWsProducers>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(ws_kernel<R, PACKED, MODE, kWsProducers>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
 }
 
 // Warp-specialised form of a narrow launch (see ws_kernel).
-template <bool PACKED, int MODE>
+template <typename R, bool PACKED, int MODE>
 cudaError_t launch_ws_t(const Batch &b, const State &s, const Hist &h, const Ckpt &c, const Noise &nz,
                         const KeyParam &kp, unsigned grid, size_t smem, int64_t g0, int64_t g1, const WaitCtl &wait,
                         cudaStream_t st) {
-    const cudaError_t e = ws_smem_limit<PACKED, MODE>(smem);
+    const cudaError_t e = ws_smem_limit<R, PACKED, MODE>(smem);
     if (e != cudaSuccess) return e;
-    ws_kernel<PACKED, MODE, kWsProducers><<<grid, 32 * (1 + kWsProducers), smem, st>>>(b, s, h, c, nz, kp, g0, g1,
+    ws_kernel<R, PACKED, MODE, kWsProducers><<<grid, 32 * (1 + kWsProducers), smem, st>>>(b, s, h, c, nz, kp, g0, g1,
                                                                                       wait);
     return cudaGetLastError();
 }
 
 // Whether `grid` blocks of the kernel fit on the GPU at once.
-template <bool PACKED, int MODE>
+template <typename R, bool PACKED, int MODE>
 cudaError_t ws_resident(unsigned grid, size_t smem, bool &fits) {
-    auto kern = ws_kernel<PACKED, MODE, kWsProducers>;
+    auto kern = ws_kernel<R, PACKED, MODE, kWsProducers>;
     int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = ws_smem_limit<PACKED, MODE>(smem);
+    cudaError_t e = ws_smem_limit<R, PACKED, MODE>(smem);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * (1 + kWsProducers), smem);
@@ -1216,7 +1237,7 @@ cudaError_t ws_resident(unsigned grid, size_t smem, bool &fits) {
 
 // Runs the launch warp-specialised (taken = true), unless the plan's width is over 32
 // and the 32-thread stepping blocks would not all fit on the GPU at once.
-template <int MODE>
+template <typename R, int MODE>
 cudaError_t launch_ws(const Batch &b0, const State &s, const Hist &h, const Ckpt &c, const Noise &nz, int64_t g0,
                       int64_t g1, const WaitCtl &wait, cudaStream_t st, bool &taken) {
     // 32 stepping threads per block whatever width w the plan chose (w divides the
@@ -1225,7 +1246,7 @@ cudaError_t launch_ws(const Batch &b0, const State &s, const Hist &h, const Ckpt
     Batch b = b0;
     b.sub_single = b0.sub_single * (b0.narrow / 32);
     b.sub_packed = b0.sub_packed * (b0.narrow / 32);
-    const size_t ring = sizeof(float2) * (size_t)kWsSlots * kWsSlotSteps * 32;
+    const size_t ring = sizeof(typename WsNoise<R>::T) * (size_t)kWsSlots * kWsSlotSteps * 32;
     const size_t hist = (hist_smem(h) + 15) & ~(size_t)15;
     const unsigned grid_s = (unsigned)(b.n_single * b.sub_single);
     const unsigned grid_p = (unsigned)((b.n_tiles - b.n_single) * b.sub_packed);
@@ -1233,15 +1254,15 @@ cudaError_t launch_ws(const Batch &b0, const State &s, const Hist &h, const Ckpt
     taken = true;
     if (b0.narrow > 32) {
         bool fits = true;
-        if (grid_s > 0) e = ws_resident<false, MODE>(grid_s, hist + ring, fits);
-        if (e == cudaSuccess && fits && grid_p > 0) e = ws_resident<true, MODE>(grid_p, ring, fits);
+        if (grid_s > 0) e = ws_resident<R, false, MODE>(grid_s, hist + ring, fits);
+        if (e == cudaSuccess && fits && grid_p > 0) e = ws_resident<R, true, MODE>(grid_p, ring, fits);
         if (e != cudaSuccess) return e;
         taken = fits;
         if (!fits) return cudaSuccess;
     }
     const KeyParam kp = key_param(nz.k0, nz.k1);
-    if (grid_s > 0) e = launch_ws_t<false, MODE>(b, s, h, c, nz, kp, grid_s, hist + ring, g0, g1, wait, st);
-    if (e == cudaSuccess && grid_p > 0) e = launch_ws_t<true, MODE>(b, s, h, c, nz, kp, grid_p, ring, g0, g1, wait, st);
+    if (grid_s > 0) e = launch_ws_t<R, false, MODE>(b, s, h, c, nz, kp, grid_s, hist + ring, g0, g1, wait, st);
+    if (e == cudaSuccess && grid_p > 0) e = launch_ws_t<R, true, MODE>(b, s, h, c, nz, kp, grid_p, ring, g0, g1, wait, st);
     return e;
 }
 
@@ -1254,10 +1275,10 @@ cudaError_t launch_integrate_t(const Batch &b, const State &s, const Hist &h, co
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    if constexpr (sizeof(R) == 4 && PPT == 1 && ABP_WS) {
+    if constexpr (PPT == 1 && ABP_WS) {
         if (b.narrow > 0 && b.narrow <= ABP_WS_WIDEST && wait && wait->status) {
             bool taken = false;
-            const cudaError_t e = launch_ws<MODE>(b, s, h, c, nz, g0, g1, *wait, st, taken);
+            const cudaError_t e = launch_ws<R, MODE>(b, s, h, c, nz, g0, g1, *wait, st, taken);
             if (e != cudaSuccess || taken) return e;
         }
     }
@@ -1307,7 +1328,7 @@ cudaError_t launch_integrate(const Batch &b, const State &s, const Hist &h, cons
     if (b.narrow) ppt = 1;
     if (s.fp64) {
         switch (ppt) {
-            case 1: return launch_integrate_t<double, 1>(b, s, h, c, nz, g0, g1, st);
+            case 1: return launch_integrate_t<double, 1>(b, s, h, c, nz, g0, g1, st, wait);
             case 2: return launch_integrate_t<double, 2>(b, s, h, c, nz, g0, g1, st);
             case 4: return launch_integrate_t<double, 4>(b, s, h, c, nz, g0, g1, st);
         }
