@@ -1251,11 +1251,13 @@ abp_status abp_reset(abp_ctx *ctx, uint64_t seed) {
     if (ctx->live_stream) cudaStreamSynchronize(ctx->live_stream);  // copies of the previous run end first
     ctx->live_sent = ctx->live_ready = 0;
     cudaStream_t s = ctx->stream;
-    cudaError_t e = cudaMemsetAsync(ctx->d_status.p, 0, sizeof(int32_t), s);
+    cudaError_t e = cudaSuccess;
+    int32_t *const status = (int32_t *)ctx->d_status.p;  // cleared by the initial condition's kernel, if any
+    if (ctx->n_tiles == 0) e = cudaMemsetAsync(status, 0, sizeof(int32_t), s);
     if (e == cudaSuccess && ctx->d_hx.bytes) e = cudaMemsetAsync(ctx->d_hx.p, 0, ctx->d_hx.bytes, s);
     if (e == cudaSuccess && ctx->d_hv.bytes) e = cudaMemsetAsync(ctx->d_hv.p, 0, ctx->d_hv.bytes, s);
     if (e == cudaSuccess) {
-        e = launch_init(ctx->batch(), ctx->state(), ctx->hist(), ctx->ckpt(), ctx->noise(), s);
+        e = launch_init(ctx->batch(), ctx->state(), ctx->hist(), ctx->ckpt(), ctx->noise(), s, status);
         ctx->launches += ctx->n_tiles > 0 ? 1 : 0;
     }
     return e == cudaSuccess ? ABP_OK : cuda_fail(ctx, e, "reset");
@@ -1416,9 +1418,8 @@ abp_status send_snapshot(abp_ctx *ctx, int64_t k) {
     const size_t ns = (size_t)ctx->n_sets;
     double *dmom = ctx->live_mom ? (double *)ctx->d_live_mom.p + (size_t)k * ns * 8 : nullptr;
     if (dmom) {
-        e = launch_reduce(ctx->batch(), ctx->state(), ctx->noise(), ctx->g, (double *)ctx->d_partials.p, dmom, s);
-        ctx->launches += (ctx->n_sets > 0 && ctx->n_single > 0 ? 1 : 0) + (ctx->n_unpacked > 0 ? 1 : 0) +
-                         (ctx->n_sets > ctx->n_unpacked ? 1 : 0);
+        e = launch_reduce(ctx->batch(), ctx->state(), ctx->noise(), ctx->g, (double *)ctx->d_partials.p, dmom, s,
+                          &ctx->launches);
     }
     if (e == cudaSuccess) e = cudaEventRecord(ctx->live_done[slot], s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(ls, ctx->live_done[slot], 0);
@@ -1669,10 +1670,8 @@ abp_status abp_reduce(abp_ctx *ctx, double *moments, uint32_t *hist_x, uint32_t 
         if (copy) dst = (double *)ctx->d_moments.p;
         if (k == PtrKind::Host && !copy) synced = true;
         cudaError_t e = launch_reduce(ctx->batch(), ctx->state(), ctx->noise(), ctx->g, (double *)ctx->d_partials.p,
-                                      dst, ctx->stream);
+                                      dst, ctx->stream, &ctx->launches);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "reduction launch");
-        ctx->launches += (ctx->n_sets > 0 && ctx->n_single > 0 ? 1 : 0) + (ctx->n_unpacked > 0 ? 1 : 0) +
-                         (ctx->n_sets > ctx->n_unpacked ? 1 : 0);
         if (copy && (st = deliver(ctx, moments, ctx->d_moments.p, bytes, &synced)) != ABP_OK) return st;
     }
     if (hist_x && ctx->d_hx.bytes)

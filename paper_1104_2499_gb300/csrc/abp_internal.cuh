@@ -148,12 +148,22 @@ __host__ __device__ inline double mom_sub(double x, double y) {
 #endif
 }
 __host__ __device__ inline void moments_from_sums(double *o, const double *a, int64_t M, int64_t n, double dt) {
+    const double T = mom_mul((double)n, dt);
+    if (M == 1) {
+        // x / 1 = x and no spread: one division instead of five (an FP64 division takes
+        // some 550 cycles on this GPU, and one-trajectory sets are the paper's work items)
+        o[0] = a[0];
+        o[1] = 0.0;
+        o[2] = a[3];
+        o[3] = T > 0.0 ? mom_sub(a[3], mom_mul(a[2], a[2])) / mom_mul(2.0, T) : 0.0;
+        for (int j = 0; j < 4; ++j) o[4 + j] = a[j];
+        return;
+    }
     const double Md = (double)M;
     const double mean_v = M > 0 ? a[0] / Md : 0.0;
     const double var_v = M > 1 ? mom_sub(a[1], mom_mul(mom_mul(Md, mean_v), mean_v)) / (Md - 1.0) : 0.0;
     const double msd = M > 0 ? a[3] / Md : 0.0;
     const double mdx = M > 0 ? a[2] / Md : 0.0;
-    const double T = mom_mul((double)n, dt);
     o[0] = mean_v;
     o[1] = M > 0 ? sqrt((var_v > 0.0 ? var_v : 0.0) / Md) : 0.0;
     o[2] = msd;
@@ -202,8 +212,10 @@ inline int current_device() {
 cudaError_t launch_combine_moments(int32_t n, double *moments, const int64_t *M, const int64_t *N, double dt,
                                    cudaStream_t st);
 
+// status (may be NULL): the context's status word, cleared by the kernel (not when the
+// batch has no tiles: nothing is launched then).
 cudaError_t launch_init(const Batch &b, const State &s, const Hist &h, const Ckpt &c, const Noise &nz,
-                        cudaStream_t st);
+                        cudaStream_t st, int32_t *status = nullptr);
 // NVTX range over one C ABI call (nested ranges of the calling thread), for
 // profilers that trace the host timeline; without a tool attached the push
 // and pop return at once.
@@ -224,7 +236,6 @@ struct WaitCtl {
 
 cudaError_t launch_integrate(const Batch &b, const State &s, const Hist &h, const Ckpt &c, const Noise &nz,
                              int ppt, int64_t g0, int64_t g1, cudaStream_t st, const WaitCtl *wait = nullptr);
-// partials: [n_tiles][4] scratch; moments: [n_sets][8].
 // The per-set coefficient tables of a batch in one device buffer of coef_table_bytes(n)
 // bytes: coef_tables gives the two tables inside it, launch_coef fills them from the
 // device parameter array (the step's FP64 set-up done once per batch instead of at the
@@ -233,8 +244,9 @@ size_t coef_table_bytes(int32_t n_sets);
 void coef_tables(void *buf, int32_t n_sets, const void **coef_f, const void **coef_d);
 cudaError_t launch_coef(const abp_params *params, int32_t n_sets, double dt, void *buf, cudaStream_t st);
 
+// partials: [n_tiles][4] scratch; moments: [n_sets][8]; *kernels: launches added.
 cudaError_t launch_reduce(const Batch &b, const State &s, const Noise &nz, int64_t g, double *partials,
-                          double *moments, cudaStream_t st);
+                          double *moments, cudaStream_t st, int64_t *kernels = nullptr);
 cudaError_t launch_get_state(const Batch &b, const State &s, double dt, int64_t g, double *x, double *x0, double *v,
                              double *e, double *vbar, cudaStream_t st);
 cudaError_t launch_philox(uint32_t k0, uint32_t k1, const uint64_t *traj, const uint64_t *m, int64_t n,
