@@ -590,13 +590,13 @@ bool plan_tiles(int32_t n_sets, const int64_t *n_traj, const int64_t *n_steps, i
     // one trajectory per thread: u1 = ceil(W / schedulers) with one trajectory per thread
     // in narrow blocks, 2 ceil(tiles / SMs) in blocks of a whole tile, u2 = 2 ceil(W2 /
     // schedulers) with two (W, W2: warps of 32, of 64 trajectories).  Measured on
-    // one-trajectory sets, 2,000 Euler-Maruyama steps: about 41 u1 + 30 us in blocks of 64
-    // threads (32: the same), 41.3 u + 23 in whole tiles, 38.1 u2 + 29 with two per thread
-    // (any block width); Heun 64 and 61 us per unit.  So two per thread where 0.93 u2 <= u1:
-    // 228 tiles 154 us (u1 = 3) against 178 (u2 = 4) and 189 (whole tiles, before), 256
-    // tiles 179 against 197 and 189, 460 tiles 322 against 334 and 354, 2,000 tiles 1,090
-    // against 1,139 and 1,172.  With xorshift noise two per thread is slower (256 tiles 198
-    // against 178 us), the FP64 state has no paired instructions: one.
+    // one-trajectory sets, 2,000 Euler-Maruyama steps: about 40.4 u1 + 17 us in blocks of 64
+    // threads (32: the same) and 38.1 u2 + 29 with two per thread (any block width); Heun 63
+    // and 61 us per unit.  So two per thread where 0.93 u2 <= u1: 228 tiles 137 us (u1 = 3)
+    // against 178 (u2 = 4), 380 tiles 219 against 258, 1,000 tiles 562 against 583.  One
+    // 256-thread block per tile, as before, took 189, 275 and 601 us.  With xorshift noise
+    // two per thread is slower (256 tiles 198 against 178 us), the FP64 state has no paired
+    // instructions: one.
     p.packed_ppt = 1;
     p.packed_threads = p.narrow ? p.narrow : kThreads;
     if (p.narrow == 0 && n_tiles > p.n_single) {

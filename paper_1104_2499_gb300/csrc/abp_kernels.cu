@@ -361,9 +361,9 @@ __device__ __forceinline__ void group_step(const Coefs<R, PPT, OWN> &ks, const R
 // the compiler interleaves them.  FP32 Euler-Maruyama at two trajectories per thread
 // takes 8 blocks: 2,048 sets x 20,000 steps in 38.1 ms on the work queue (6: 39.4 ms, 10:
 // 38.9) and 38.5 ms lockstep.  Stochastic Heun takes 4 (512 sets x 10^4 steps 7.67 ms;
-// 2: 7.75, 3: 7.78, 6: 7.76), xorshift 8 (4.91 ms; 4: 4.93, 2: 5.04).  The other FP32
-// kernels take 4: one trajectory per thread 41.8 ms (2: 42.4, 1: 44.9), four 38.9 ms
-// (2: 40.2).  The FP64 kernels keep 2, longer bodies spill.
+// 2: 7.75, 3: 7.78, 6: 7.76), xorshift 8 (4.91 ms; 4: 4.93, 2: 5.04).  FP32 at one
+// trajectory per thread takes 8 with the registers of min_blocks below, four trajectories
+// per thread 4 (2,048 sets 38.9 ms, 2: 40.2).  The FP64 kernels keep 2, longer bodies spill.
 #ifndef ABP_UNROLL_EM2
 #define ABP_UNROLL_EM2 8
 #endif
@@ -375,6 +375,9 @@ __device__ __forceinline__ void group_step(const Coefs<R, PPT, OWN> &ks, const R
 #endif
 #ifndef ABP_UNROLL_XS2
 #define ABP_UNROLL_XS2 8
+#endif
+#ifndef ABP_UNROLL_1
+#define ABP_UNROLL_1 8
 #endif
 template <typename R, int PPT, int MODE, bool QUEUE, bool PACKED = false>
 constexpr int group_unroll() {
@@ -388,6 +391,8 @@ constexpr int group_unroll() {
         return ABP_UNROLL_XS2;
     else if constexpr (sizeof(R) == 8)
         return 2;
+    else if constexpr (PPT == 1)
+        return ABP_UNROLL_1;
     else
         return kGroupUnroll;
 }
@@ -395,13 +400,21 @@ constexpr int group_unroll() {
 // Resident blocks per SM asked of the compiler (bounds its registers; 0: its own choice).
 // The xorshift kernels at two trajectories per thread take four (64 registers, no
 // spills): 512 x 1,024 trajectories x 10^4 steps in 4.91 ms against 5.13 ms (work queue)
-// and 5.30 ms (lockstep) with three.  The others gain nothing from it (Euler-Maruyama
-// 38.4-39.3 ms against 38.0, Heun 7.80 against 7.65: not bound by latency).
+// and 5.30 ms (lockstep) with three.  The others at two or four gain nothing from it
+// (Euler-Maruyama 38.4-39.3 ms against 38.0, Heun 7.80 against 7.65: not bound by latency).
+// The kernels at one trajectory per thread serve the batches that put one or two warps
+// on a scheduler and are bound by their latency: told that four blocks are enough the
+// compiler takes up to 64 registers instead of 56 and overlaps more of the chain (36,692
+// one-trajectory sets x 3,164 steps 191 -> 146 us, 20,000 trajectories of one set x 1,659
+// steps 88 -> 82 us, 53 sets of 829 on the work queue 557 -> 488 us).  Two or three blocks
+// are no faster there, and slower where tiles are nearly empty and blocks per SM count
+// (2,000 sets of 20 on the work queue: 471 us, 859 and 599 with two and three).
 #ifndef ABP_BLOCKS_XS2
 #define ABP_BLOCKS_XS2 4
 #endif
 template <typename R, int PPT, int MODE, bool PACKED = false>
 constexpr int min_blocks() {
+    if (sizeof(R) == 4 && PPT == 1) return 4;
     return !PACKED && sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift ? ABP_BLOCKS_XS2 : 0;
 }
 
@@ -843,9 +856,11 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
                 for (int i = 0; i < 4; ++i) out[(4 * j + i) * 32] = z[i];
             }
         } else {
-            // two counter blocks at a time: a producer with its scheduler to itself is bound by
-            // the latency of a block's chain
-#pragma unroll 2
+            // Euler-Maruyama takes two counter blocks at a time: a producer is bound by the latency
+            // of a block's chain (16,384 trajectories x 3,000 steps 99 -> 94 us); with Heun, whose
+            // stepping warps need the issue slots, one (159 -> 149)
+            constexpr int U = MODE == kModeHeun ? 1 : 2;
+#pragma unroll U
             for (int j = p; j < SS / 4; j += NP) {
                 const uint4 wv = step_block((uint32_t)(a * (SS / 4) + j), ss, K);
                 float nr, cs, sn;
