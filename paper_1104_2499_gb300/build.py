@@ -20,7 +20,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "_build")
 LIB = os.path.join(OUT, "libabp.so")
 SOURCES = ["abp_api.cu", "abp_kernels.cu", "abp_adjoint.cu", "abp_noalloc.cu"]
-HEADERS = ["abp_device.cuh", "abp_internal.cuh", "abp_ctx.cuh"]
+HEADERS = ["abp_device.cuh", "abp_internal.cuh", "abp_ctx.cuh", "abp_cos_table.inc"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

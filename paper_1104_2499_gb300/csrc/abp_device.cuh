@@ -193,6 +193,85 @@ __device__ __forceinline__ void box_muller_f64(uint32_t wa, uint32_t wb, double 
 }
 
 // --------------------------------------------------------------------------
+// FP64 cosine and sine of 2 pi t for the FP64 state.  FP64 is slow on this GPU (a warp
+// instruction holds the SM's pipe 16 cycles, a dependent one waits 55), and cospi /
+// sincospi spend some 25 / 45 of them; here t is split as k / 1024 + f, |f| <= 2^-11, and
+// the angle sums formed from a table of cos(2 pi k / 1024) in two doubles and short
+// Taylor polynomials in f (the dropped terms are below 2^-59): 13 for the cosine, 15 for
+// both.  The last addition is the only one whose rounding counts: measured against 112-bit
+// values, error at most 5.7e-17 and 2.7e-17 r.m.s. (cospi and sincospi: 1.3e-16 and
+// 3.2e-17).  4,096 trajectories x 1,000 steps, bound by the stepping warp's chain: 1,103 ->
+// 879 us; 20,000 trajectories, bound by the FP64 pipe: 4.64 -> 3.79 ms.  (Whole periods
+// taken off first by rint instead of the branch below: 978 us.)
+static __device__ const double2 kCos1024[257] = {
+#include "abp_cos_table.inc"
+};
+
+// sin(2 pi f) and cos(2 pi f) - 1.
+__device__ __forceinline__ void small_angle(double f, double &s, double &c) {
+    const double f2 = f * f;
+    s = fma(f * f2, fma(f2, 0x1.466bc6775aae2p+6, -0x1.4abbce625be53p+5), f * 0x1.921fb54442d18p+2);
+    c = f2 * fma(f2, 0x1.03c1f081b5ac4p+6, -0x1.3bd3cc9be45dep+4);
+}
+
+// x with its sign changed where bit 31 of m is set.
+__device__ __forceinline__ double flip(double x, uint32_t m) {
+    return __hiloint2double(__double2hiint(x) ^ (int)(m & 0x80000000u), __double2loint(x));
+}
+
+// Table entries of angle k (mod 1024): cos and sin of its place in the first quadrant, and
+// what the quadrant changes: the sign of the sine of the small angle (odd) and of the cosine.
+struct TableAngle {
+    double2 c, s;
+    uint32_t odd, neg_c, neg_s;
+    __device__ __forceinline__ explicit TableAngle(uint32_t k) {
+        const uint32_t j = k & 255u, q = (k >> 8) & 3u;
+        const uint32_t i = q & 1u ? 256u - j : j;
+        c = __ldg(&kCos1024[i]);
+        s = __ldg(&kCos1024[256u - i]);
+        odd = q << 31;
+        neg_c = (q + 1u) << 30;
+        neg_s = q << 30;
+    }
+};
+
+__device__ __forceinline__ double cos_2pi(double t) {
+    // beyond 2^40 periods (a diverged trajectory) and for non-finite t: the general function
+    if ((uint32_t)(__double2hiint(t) & 0x7fffffff) >= 0x42700000u) return cospi(2.0 * t);
+    const double big = 0x1.8p+52;
+    const double m = fma(t, 1024.0, big);  // the nearest integer k in its low bits
+    const double f = fma(m - big, -0x1p-10, t);
+    const TableAngle a((uint32_t)__double2loint(m));
+    double s, c;
+    small_angle(f, s, c);
+    const double r = a.c.x + fma(-a.s.x, flip(s, a.odd), fma(a.c.x, c, a.c.y));
+    return flip(r, a.neg_c);
+}
+
+// cos and sin of 2 pi u for u = n 2^-23.
+__device__ __forceinline__ void sincos_2pi_u23(uint32_t n, double &sn, double &cs) {
+    const uint32_t r = n + 4096u;  // u = k / 1024 + f, f in [-2^-11, 2^-11)
+    const double f = (double)((int)(r & 8191u) - 4096) * 0x1p-23;
+    const TableAngle a(r >> 13);
+    double s, c;
+    small_angle(f, s, c);
+    s = flip(s, a.odd);
+    cs = flip(a.c.x + fma(-a.s.x, s, fma(a.c.x, c, a.c.y)), a.neg_c);
+    sn = flip(a.s.x + fma(a.c.x, s, fma(a.s.x, c, a.s.y)), a.neg_s);
+}
+
+// Box-Muller of one word pair for the steps of the FP64 state (the mapping of
+// box_muller_f64, which the initial velocity keeps).
+__device__ __forceinline__ void box_muller_step_f64(uint32_t wa, uint32_t wb, double &z_even, double &z_odd) {
+    const double u1 = ((double)wa + 0.5) * 0x1p-32;
+    const double r = sqrt(-2.0 * log(u1));
+    double s, c;
+    sincos_2pi_u23(wb >> 9, s, c);
+    z_even = r * c;
+    z_odd = r * s;
+}
+
+// --------------------------------------------------------------------------
 // Per-set coefficients of the Euler-Maruyama map, built once per thread from
 // the set's parameters.  With K = dt h 0.453 (2 pi / L) and c = cos phi,
 //   -U'(x) dt = K (c + 2a cos 2phi) = K c + 4 a K c^2 - 2 a K      (Eq. (pot))
@@ -264,10 +343,9 @@ __device__ __forceinline__ Coef<R> load_coef(const void *table, const abp_params
     return make_coef<R>(p.q, p.c, p.d, p.gamma0, p.F0, p.D, p.h, p.L, p.asym, dt);
 }
 
-__device__ __forceinline__ float cos_phase(float y) {
-    return __cosf(fmaf(y, kTwoPiF, (float)(2.0 * kPi * kPhaseShifted)));
-}
-__device__ __forceinline__ double cos_phase(double y) { return cospi(2.0 * (y + kPhase)); }
+// The FP64 force's cos phi at position fraction y + yacc; y + kPhase changes only at the
+// folds, so it is off the step's chain.
+__device__ __forceinline__ double cos_phase(double y, double yacc) { return cos_2pi(yacc + (y + kPhase)); }
 
 // FP32 phase of the force at position fraction y + yacc.  The fraction y only
 // changes at the folds, so the integrator keeps pb = phase_base(y) beside it
@@ -277,11 +355,12 @@ __device__ __forceinline__ float phase_base(float y) {
 }
 __device__ __forceinline__ float phase_arg(float pb, float yacc) { return fmaf(yacc, kTwoPiF, pb); }
 
-// One Euler-Maruyama step with the normal z_n; every right-hand side uses the step-n
-// values.
-template <typename R>
-__device__ __forceinline__ void em_step(const Coef<R> &k, R z, R y, R &yacc, R &v, R &e) {
-    const R cphi = cos_phase(y + yacc);
+// One Euler-Maruyama step of the FP64 state with the normal z_n; every right-hand side
+// uses the step-n values.
+__device__ __forceinline__ void em_step_f64(const Coef<double> &k, double z, double y, double &yacc, double &v,
+                                            double &e) {
+    using R = double;
+    const R cphi = cos_phase(y, yacc);
     const R t1 = fma(-k.Bd, v * v, k.A);
     const R hv = fma(k.Bd, e, k.Gd);
     const R a1 = fma(k.sigma, z, k.F);
@@ -474,9 +553,9 @@ __device__ __forceinline__ float normal_from_block_f32(uint4 w, uint32_t k) {
 __device__ __forceinline__ double normal_from_block_f64(uint4 w, uint32_t k) {
     double ze, zo;
     if (k < 2)
-        box_muller_f64(w.x, w.y, ze, zo);
+        box_muller_step_f64(w.x, w.y, ze, zo);
     else
-        box_muller_f64(w.z, w.w, ze, zo);
+        box_muller_step_f64(w.z, w.w, ze, zo);
     return (k & 1) ? zo : ze;
 }
 

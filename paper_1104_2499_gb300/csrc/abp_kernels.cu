@@ -290,7 +290,7 @@ __device__ __forceinline__ void single_step(const Coefs<R, PPT, OWN> &ks, const 
             step_f32<MODE == kModeHeun>(k, nrs, (j & 1) ? sn : cs, S.pb[q], S.yacc[q], S.v[q], S.e[q]);
         } else {
             const double z = normal_from_block_f64(w, j);
-            em_step<double>(k, z, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step_f64(k, z, S.y[q], S.yacc[q], S.v[q], S.e[q]);
         }
     }
 }
@@ -350,12 +350,12 @@ __device__ __forceinline__ void group_step(const Coefs<R, PPT, OWN> &ks, const R
         for (int q = 0; q < PPT; ++q) {
             const Coef<R> &k = ks.of(q);
             double z0, z1, z2, z3;
-            box_muller_f64(w[q].x, w[q].y, z0, z1);
-            box_muller_f64(w[q].z, w[q].w, z2, z3);
-            em_step<double>(k, z0, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, z1, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, z2, S.y[q], S.yacc[q], S.v[q], S.e[q]);
-            em_step<double>(k, z3, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            box_muller_step_f64(w[q].x, w[q].y, z0, z1);
+            box_muller_step_f64(w[q].z, w[q].w, z2, z3);
+            em_step_f64(k, z0, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step_f64(k, z1, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step_f64(k, z2, S.y[q], S.yacc[q], S.v[q], S.e[q]);
+            em_step_f64(k, z3, S.y[q], S.yacc[q], S.v[q], S.e[q]);
         }
     }
 }
@@ -572,7 +572,7 @@ __device__ __forceinline__ void advance_ws(const Coef<R> &k, Slots<R, 1> &S, int
         if constexpr (sizeof(R) == 4)
             step_f32<HEUN>(k, t.x, t.y, S.pb[0], S.yacc[0], S.v[0], S.e[0]);
         else
-            em_step<double>(k, t, S.y[0], S.yacc[0], S.v[0], S.e[0]);
+            em_step_f64(k, t, S.y[0], S.yacc[0], S.v[0], S.e[0]);
     };
     while (n < n_end) {
         const int64_t a = n / SS;
@@ -857,8 +857,8 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
             for (int j = p; j < SS / 4; j += NP) {
                 const uint4 wv = step_block((uint32_t)(a * (SS / 4) + j), ss, K);
                 double z[4];
-                box_muller_f64(wv.x, wv.y, z[0], z[1]);
-                box_muller_f64(wv.z, wv.w, z[2], z[3]);
+                box_muller_step_f64(wv.x, wv.y, z[0], z[1]);
+                box_muller_step_f64(wv.z, wv.w, z[2], z[3]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) out[(4 * j + i) * 32] = z[i];
             }

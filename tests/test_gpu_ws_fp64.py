@@ -66,3 +66,13 @@ def test_fp64_packed_items_and_timeout(abp):
         ens.integrate()
         ens.synchronize()
         np.testing.assert_array_equal(ens.state(host=True)["x"].numpy(), sb["x"].cpu().numpy())
+
+
+def test_fp64_positions_far_beyond_the_table_range(abp):
+    # a free particle driven to 10^15 periods a step: the force's cosine stays bounded, so the
+    # velocity is the driven one (the potential adds at most 3e-3 a step)
+    w = W.Workload(name="far", sets=[W.params(D=0.0, d=0.0, gamma0=0.0, F0=1e18)], n_traj=[40], n_steps=[100], dt=1e-3,
+                   seed=2)
+    st = run(abp, w, schedule=1, steps_per_launch=1000)[1]
+    np.testing.assert_allclose(st["v"].cpu().numpy(), 1e18 * 1e-3 * 100, rtol=1e-13)
+    assert bool(torch.isfinite(st["x"]).all())
