@@ -94,9 +94,10 @@ struct AdjArgs {
     Ckpt ck;
     Noise nz;
     RoundKeys K;        // Philox round keys of the seed (constant bank)
-    float4 *sub;        // [n_sub][total_traj] sub-checkpoints (scratch)
+    float4 *sub;        // [per][n_sub][total_traj] sub-checkpoints (scratch)
     int64_t n_sub;      // sub-checkpoint slots per segment (sub_slots)
-    uint4 *words;       // [block][n_blk][2][threads] noise hand-off of the segment (scratch), WORDS kernels only
+    int per;            // segments per launch (segments_per_launch)
+    uint4 *words;       // [block][per][n_blk][2][threads] noise hand-off of the launch (scratch), WORDS kernels only
     int64_t n_blk;      // Philox blocks per segment (kSub / 4 per sub-checkpoint slot)
     int tile0;          // first tile of the launch (its group of tiles)
     const double *w;    // [n_sets] dJ/dmean_v, NULL = 1
@@ -236,7 +237,7 @@ __device__ __forceinline__ void block_sum6(double (&a)[6], double (*red)[6]) {
 // (y, yacc, v, e) = c0, leaving the state at the start of each chunk in the
 // sub-checkpoint scratch.  Whole chunks take their noise one Philox block per four
 // steps (the forward's own path); partial ones step one at a time.
-__device__ __forceinline__ void level1_segment(const AdjArgs &a, const Coef<float> &k, const StepStream &ss,
+__device__ __forceinline__ void level1_segment(const AdjArgs &a, float4 *slots, const Coef<float> &k, const StepStream &ss,
                                                int64_t idx, int64_t s0, int64_t s1, float4 c0) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
@@ -247,7 +248,7 @@ __device__ __forceinline__ void level1_segment(const AdjArgs &a, const Coef<floa
     nc.m = 0;
     for (int j = 0; j < seg.n; ++j) {
         const int64_t n0 = seg.begin(j);
-        a.sub[(size_t)dchk(j, a.n_sub, a.b.dbg) * T + idx] = make_float4(y, yacc, v, e);
+        slots[(size_t)dchk(j, a.n_sub, a.b.dbg) * T + idx] = make_float4(y, yacc, v, e);
         if (seg.whole(j)) {
 #pragma unroll
             for (int b2 = 0; b2 < kSub / 4; ++b2) {
@@ -305,20 +306,19 @@ __device__ __forceinline__ void pair_blocks(uint32_t m, const StepStream (&ss)[2
 }
 
 template <bool WORDS>
-__device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<float> &k, const StepStream (&ss)[2],
-                                                const int64_t (&idx)[2], bool store1, int64_t s0, int64_t s1,
-                                                float4 c0, float4 c1, int block) {
+__device__ __forceinline__ void level1_segment2(const AdjArgs &a, float4 *slots, uint4 *wp, const Coef<float> &k,
+                                                const StepStream (&ss)[2], const int64_t (&idx)[2], bool store1,
+                                                int64_t s0, int64_t s1, float4 c0, float4 c1) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
-    uint4 *const wp = WORDS ? a.words + (size_t)block * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x : nullptr;
     float y[2] = {c0.x, c1.x};
     float2 Y = make_float2(c0.y, c1.y), V = make_float2(c0.z, c1.z), E = make_float2(c0.w, c1.w);
     float2 PB = make_float2(phase_base(y[0]), phase_base(y[1]));
     const Coef2 k2 = make_coef2(k);
     auto store = [&](int j) {
         const size_t js = (size_t)dchk(j, a.n_sub, a.b.dbg);
-        a.sub[js * T + idx[0]] = make_float4(y[0], Y.x, V.x, E.x);
-        if (store1) a.sub[js * T + idx[1]] = make_float4(y[1], Y.y, V.y, E.y);
+        slots[js * T + idx[0]] = make_float4(y[0], Y.x, V.x, E.x);
+        if (store1) slots[js * T + idx[1]] = make_float4(y[1], Y.y, V.y, E.y);
     };
     auto whole_chunk = [&](int j) {
         const int64_t n0 = (seg.c0 + j) * kSub;
@@ -380,20 +380,20 @@ __device__ __forceinline__ void level1_segment2(const AdjArgs &a, const Coef<flo
 // reverse order, each re-run from its sub-checkpoint into registers and swept
 // backwards.  Each chunk's sub-checkpoint is loaded one chunk ahead, so its
 // memory latency overlaps the previous chunk's arithmetic.
-__device__ __forceinline__ void reverse_chunks(const AdjArgs &a, const Coef<float> &k, const StepStream &ss, float kx,
-                                               float dtf, int64_t idx, int64_t s0, int64_t s1, float &lx, float &lv,
+__device__ __forceinline__ void reverse_chunks(const AdjArgs &a, const float4 *slots, const Coef<float> &k,
+                                               const StepStream &ss, float kx, float dtf, int64_t idx, int64_t s0, int64_t s1, float &lx, float &lv,
                                                float &le, float (&acc)[6]) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
     NoiseCursor nc;
     nc.valid = false;
     nc.m = 0;
-    float4 c_next = a.sub[(size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg) * T + idx];
+    float4 c_next = slots[(size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg) * T + idx];
     for (int j = seg.n - 1; j >= 0; --j) {
         const int64_t n0 = seg.begin(j);
         const int len = (int)(seg.end(j) - n0);
         const float4 cj = c_next;
-        if (j > 0) c_next = a.sub[(size_t)dchk(j - 1, a.n_sub, a.b.dbg) * T + idx];
+        if (j > 0) c_next = slots[(size_t)dchk(j - 1, a.n_sub, a.b.dbg) * T + idx];
         float y = cj.x, yacc = cj.y, v = cj.z, e = cj.w;
         float pb = phase_base(y);
         float ys[kSub], vs[kSub], es[kSub], szs[kSub];  // ys: the force phase of each step
@@ -492,10 +492,10 @@ __device__ __forceinline__ void reverse_step_x2(const RevCoef2 &c, float2 ph, fl
 typedef uint4 WordStage[kSub / 4][2][kRevPairThreads];
 
 template <bool WORDS>
-__device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<float> &k, const StepStream (&ss)[2],
-                                                float kx, float dtf, const int64_t (&idx)[2], int64_t s0, int64_t s1,
-                                                float2 &lx, float2 &lv, float2 &le, float2 (&acc)[6],
-                                                WordStage *stage, int block) {
+__device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const float4 *slots, const uint4 *wr,
+                                                const Coef<float> &k, const StepStream (&ss)[2], float kx, float dtf,
+                                                const int64_t (&idx)[2], int64_t s0, int64_t s1, float2 &lx,
+                                                float2 &lv, float2 &le, float2 (&acc)[6], WordStage *stage) {
     const int64_t T = a.b.total_traj;
     const SegChunks seg(s0, s1);
     const int j0w = seg.first_whole(), j1w = seg.last_whole();  // chunks [j0w, j1w) are whole
@@ -503,8 +503,6 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     const RevCoef2 rc = make_rev_coef2(k, kx, dtf);
     // WORDS: copy whole chunk jj's blocks into stage[jj % kStages]; one commit group per
     // call, empty for chunks that are not whole, so that groups and chunks stay in step
-    const uint4 *const wr =
-        WORDS ? a.words + (size_t)block * (size_t)a.n_blk * (2 * kRevPairThreads) + threadIdx.x : nullptr;
     auto fetch = [&](int jj) {
         if (jj >= j0w && jj < j1w) {
             WordStage &st = stage[jj % kStages];
@@ -521,13 +519,13 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
 #pragma unroll
         for (int i = 0; i < kStages - 1; ++i) fetch(seg.n - 1 - i);
     const size_t jl = (size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg);
-    float4 n0c = a.sub[jl * T + idx[0]], n1c = a.sub[jl * T + idx[1]];
+    float4 n0c = slots[jl * T + idx[0]], n1c = slots[jl * T + idx[1]];
     for (int j = seg.n - 1; j >= 0; --j) {
         const float4 c0 = n0c, c1 = n1c;
         if (j > 0) {
             const size_t jp = (size_t)dchk(j - 1, a.n_sub, a.b.dbg);
-            n0c = a.sub[jp * T + idx[0]];
-            n1c = a.sub[jp * T + idx[1]];
+            n0c = slots[jp * T + idx[0]];
+            n1c = slots[jp * T + idx[1]];
         }
         if (WORDS) {
             fetch(j - (kStages - 1));
@@ -627,14 +625,15 @@ __device__ __forceinline__ void reverse_chunks2(const AdjArgs &a, const Coef<flo
     }
 }
 
-// One launch per segment index, level and group of tiles, segments in reverse
-// order: level 1 (a plain forward re-run, light on registers) for segment `seg`
-// of the group's trajectories, then level 2 and the reverse sweep
-// (register-heavy) for the same segment.  The level-1 launch of segment seg - 1
-// runs on a second stream while the reverse sweep of segment seg runs, into the
-// other of two sub-checkpoint buffers.  Between launches each trajectory keeps its adjoint
+// One launch per run of consecutive segments, level and group of tiles, runs in reverse
+// order: level 1 (a plain forward re-run, light on registers) for the run's segments
+// of the group's trajectories, every segment in blocks of its own (blockIdx.y; each
+// starts from its own checkpoint), then level 2 and the reverse sweep
+// (register-heavy), the run's segments one after the other.  The level-1 launch of the
+// run before goes on a second stream while the reverse sweep of a run goes, into the
+// other of two sub-checkpoint buffers.  Between segments each trajectory keeps its adjoint
 // state lambda = (x, v, e) and its six gradient sums in global memory.
-// Trajectories of sets shorter than seg K skip.
+// Trajectories of sets shorter than a segment's start skip it.
 constexpr int kAdjGroups = abp_ctx::kAdjGroups;
 
 struct SegView {
@@ -642,10 +641,23 @@ struct SegView {
     double *G;    // [6][total_traj] gradient sums
 };
 
-// Both per-segment kernels run `sub` blocks per tile, block j of a tile taking
+// The sub-checkpoint slots and the thread's hand-off blocks of segment i of a launch.
+__device__ __forceinline__ float4 *segment_slots(const AdjArgs &a, int i) {
+    return a.sub + (size_t)i * (size_t)a.n_sub * (size_t)a.b.total_traj;
+}
+
+template <bool WORDS>
+__device__ __forceinline__ uint4 *segment_words(const AdjArgs &a, int block, int i) {
+    if (!WORDS) return nullptr;
+    return a.words + ((size_t)block * (size_t)a.per + (size_t)i) * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x;
+}
+
+// Both kernels run `sub` blocks per tile, block j of a tile taking
 // its trajectories [j blockDim, (j + 1) blockDim): one trajectory per thread.
-__global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, int64_t seg, int sub) {
+__global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, int64_t seg0, int sub) {
     const Batch &b = a.b;
+    const int64_t seg = seg0 + blockIdx.y;
+    float4 *const slots = segment_slots(a, (int)blockIdx.y);
     const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
@@ -657,14 +669,16 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, i
     if (li >= b.tile_count[tile]) return;
     const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
     const StepStream ss = step_stream((uint64_t)idx + a.nz.traj_base, a.K);
-    level1_segment(a, k, ss, idx, s0, s1, a.ck.ck[(size_t)dchk(seg, a.ck.n_slots, b.dbg) * T + idx]);
+    level1_segment(a, slots, k, ss, idx, s0, s1, a.ck.ck[(size_t)dchk(seg, a.ck.n_slots, b.dbg) * T + idx]);
 }
 
 // Level 1 with two trajectories per thread (trajectories li and li +
 // blockDim.x of the block's 2 blockDim.x), `sub` blocks per tile.
 template <bool WORDS>
-__global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs a, int64_t seg, int sub) {
+__global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs a, int64_t seg0, int sub) {
     const Batch &b = a.b;
+    const int64_t seg = seg0 + blockIdx.y;
+    float4 *const slots = segment_slots(a, (int)blockIdx.y);
     const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * 2 * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
@@ -681,21 +695,20 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs
     const StepStream ss[2] = {step_stream((uint64_t)idx[0] + a.nz.traj_base, a.K),
                               step_stream((uint64_t)idx[1] + a.nz.traj_base, a.K)};
     const int64_t slot = dchk(seg, a.ck.n_slots, b.dbg);
-    level1_segment2<WORDS>(a, k, ss, idx, second, s0, s1, a.ck.ck[(size_t)slot * T + idx[0]],
-                           a.ck.ck[(size_t)slot * T + idx[1]], a.tile0 * sub + (int)blockIdx.x);
+    level1_segment2<WORDS>(a, slots, segment_words<WORDS>(a, a.tile0 * sub + (int)blockIdx.x, (int)blockIdx.y), k, ss,
+                           idx, second, s0, s1, a.ck.ck[(size_t)slot * T + idx[0]],
+                           a.ck.ck[(size_t)slot * T + idx[1]]);
 }
 
 __global__ void __launch_bounds__(kRevThreads, ABP_ADJ_MIN_BLOCKS) adjoint_reverse_kernel(AdjArgs a, SegView sv,
-                                                                                          int64_t seg, int sub,
-                                                                                          int64_t window) {
+                                                                                          int64_t seg0, int n,
+                                                                                          int sub, int64_t window) {
     const Batch &b = a.b;
     const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
-    const int64_t s0 = seg * K;
-    if (s0 >= N) return;  // uniform over the block
-    const int64_t s1 = min(s0 + K, N);
+    if (seg0 * K >= N) return;  // uniform over the block
     const abp_params p = b.params[set];
     const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, a.nz.dt);  // the forward's own coefficients
     const float dtf = (float)a.nz.dt;
@@ -703,31 +716,33 @@ __global__ void __launch_bounds__(kRevThreads, ABP_ADJ_MIN_BLOCKS) adjoint_rever
     if (li >= b.tile_count[tile]) return;
     const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
     const StepStream ss = step_stream((uint64_t)idx + a.nz.traj_base, a.K);
-    float4 l0 = sv.lam[idx];
-    // windowed adjoint: the window ending at step (seg + 1) K starts from zero
-    if (window > 0 && ((seg + 1) * K) % window == 0) l0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float lx = l0.x, lv = l0.y, le = l0.z;
-    float acc[6] = {0, 0, 0, 0, 0, 0};
-    reverse_chunks(a, k, ss, kx, dtf, idx, s0, s1, lx, lv, le, acc);
-    sv.lam[idx] = make_float4(lx, lv, le, 0.0f);
+    for (int i = n - 1; i >= 0; --i) {
+        const int64_t seg = seg0 + i, s0 = seg * K;
+        if (s0 >= N) continue;
+        float4 l0 = sv.lam[idx];
+        // windowed adjoint: the window ending at step (seg + 1) K starts from zero
+        if (window > 0 && ((seg + 1) * K) % window == 0) l0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float lx = l0.x, lv = l0.y, le = l0.z;
+        float acc[6] = {0, 0, 0, 0, 0, 0};
+        reverse_chunks(a, segment_slots(a, i), k, ss, kx, dtf, idx, s0, min(s0 + K, N), lx, lv, le, acc);
+        sv.lam[idx] = make_float4(lx, lv, le, 0.0f);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx] += (double)acc[q];
+        for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx] += (double)acc[q];
+    }
 }
 
 // The reverse kernel with two trajectories per thread (trajectories li and
 // li + blockDim.x of the block's 2 blockDim.x), `sub` blocks per tile.
 template <bool WORDS>
-__global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) adjoint_reverse_pair_kernel(AdjArgs a, SegView sv, int64_t seg,
-                                                                               int sub, int64_t window) {
+__global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) adjoint_reverse_pair_kernel(AdjArgs a, SegView sv, int64_t seg0,
+                                                                               int n, int sub, int64_t window) {
     __shared__ WordStage stage[WORDS ? kStages : 1];
     const Batch &b = a.b;
     const int tile = a.tile0 + (int)blockIdx.x / sub;
     const int li = ((int)blockIdx.x % sub) * 2 * (int)blockDim.x + (int)threadIdx.x;
     const int set = b.tile_set[tile];
     const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
-    const int64_t s0 = seg * K;
-    if (s0 >= N) return;  // uniform over the block
-    const int64_t s1 = min(s0 + K, N);
+    if (seg0 * K >= N) return;  // uniform over the block
     const int count = b.tile_count[tile];
     if (li >= count) return;
     const abp_params p = b.params[set];
@@ -739,21 +754,25 @@ __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) 
                             dchk(b.tile_first[tile] + (second ? li + (int)blockDim.x : li), T, b.dbg)};
     const StepStream ss[2] = {step_stream((uint64_t)idx[0] + a.nz.traj_base, a.K),
                               step_stream((uint64_t)idx[1] + a.nz.traj_base, a.K)};
-    float4 l0 = sv.lam[idx[0]], l1 = sv.lam[idx[1]];
-    if (window > 0 && ((seg + 1) * K) % window == 0) l0 = l1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    float2 lx = make_float2(l0.x, l1.x), lv = make_float2(l0.y, l1.y), le = make_float2(l0.z, l1.z);
-    float2 acc[6];
+    for (int i = n - 1; i >= 0; --i) {
+        const int64_t seg = seg0 + i, s0 = seg * K;
+        if (s0 >= N) continue;
+        float4 l0 = sv.lam[idx[0]], l1 = sv.lam[idx[1]];
+        if (window > 0 && ((seg + 1) * K) % window == 0) l0 = l1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        float2 lx = make_float2(l0.x, l1.x), lv = make_float2(l0.y, l1.y), le = make_float2(l0.z, l1.z);
+        float2 acc[6];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) acc[q] = make_float2(0.0f, 0.0f);
-    reverse_chunks2<WORDS>(a, k, ss, kx, dtf, idx, s0, s1, lx, lv, le, acc, stage,
-                           a.tile0 * sub + (int)blockIdx.x);
-    sv.lam[idx[0]] = make_float4(lx.x, lv.x, le.x, 0.0f);
+        for (int q = 0; q < 6; ++q) acc[q] = make_float2(0.0f, 0.0f);
+        reverse_chunks2<WORDS>(a, segment_slots(a, i), segment_words<WORDS>(a, a.tile0 * sub + (int)blockIdx.x, i), k,
+                               ss, kx, dtf, idx, s0, min(s0 + K, N), lx, lv, le, acc, stage);
+        sv.lam[idx[0]] = make_float4(lx.x, lv.x, le.x, 0.0f);
 #pragma unroll
-    for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[0]] += (double)acc[q].x;
-    if (second) {
-        sv.lam[idx[1]] = make_float4(lx.y, lv.y, le.y, 0.0f);
+        for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[0]] += (double)acc[q].x;
+        if (second) {
+            sv.lam[idx[1]] = make_float4(lx.y, lv.y, le.y, 0.0f);
 #pragma unroll
-        for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[1]] += (double)acc[q].y;
+            for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[1]] += (double)acc[q].y;
+        }
     }
 }
 
@@ -855,13 +874,14 @@ abp_status set_err(abp_ctx *ctx, abp_status st, const char *msg, cudaError_t e =
     return st;
 }
 
-// Scratch of abp_backward, one allocation: the two sub-checkpoint buffers, the
-// tile partials, the set gradients, the weights, lambda, the per-trajectory sums
-// and, last, the two Philox-block buffers of the hand-off (0 bytes without it).
-// abp_backward_traj reads lambda and the sums of the last call at the same offsets.
+// Scratch of abp_backward, one allocation: the tile partials, the set gradients, the
+// weights, lambda, the per-trajectory sums, then the two sub-checkpoint buffers and,
+// last, the two Philox-block buffers of the hand-off (0 bytes without it), each for
+// `per` segments.  abp_backward_traj reads lambda and the sums of the last call at the
+// same offsets, which depend on neither.
 struct AdjLayout {
     size_t sub1, sub, part, grad, w, lam, g, words1, words, need;
-    size_t off_part, off_grad, off_w, off_lam, off_g, off_words;
+    size_t off_part, off_grad, off_w, off_lam, off_g, off_sub, off_words;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -877,45 +897,67 @@ int pair_blocks_per_tile(const abp_ctx *ctx, int threads) {
     return (cap + 2 * threads - 1) / (2 * threads);
 }
 
-AdjLayout adj_layout(const abp_ctx *ctx, bool words) {
+AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1) {
     AdjLayout L;
     const int64_t T = ctx->total_traj, Kc = ctx->cfg.checkpoint_every;
     const int64_t n_sub = sub_slots(Kc);
-    L.sub1 = sizeof(float4) * (size_t)n_sub * (size_t)T;
-    L.sub = 2 * align256(L.sub1);  // two buffers, alternating by segment
+    L.sub1 = sizeof(float4) * (size_t)(per * n_sub) * (size_t)T;
+    L.sub = 2 * align256(L.sub1);  // two buffers, alternating by launch
     L.part = sizeof(double) * 6 * (size_t)std::max(ctx->n_tiles, 1);
     L.grad = sizeof(double) * 6 * (size_t)std::max(ctx->n_sets, 1);
     L.w = sizeof(double) * (size_t)std::max(ctx->n_sets, 1);
     L.lam = sizeof(float4) * (size_t)std::max<int64_t>(T, 1);
     L.g = sizeof(double) * 6 * (size_t)std::max<int64_t>(T, 1);
     const size_t blocks = (size_t)ctx->n_tiles * (size_t)pair_blocks_per_tile(ctx, kL1Threads);
-    L.words1 = words ? sizeof(uint4) * blocks * (size_t)(n_sub * (kSub / 4)) * 2 * kL1Threads : 0;
+    L.words1 = words ? sizeof(uint4) * blocks * (size_t)(per * n_sub * (kSub / 4)) * 2 * kL1Threads : 0;
     L.words = 2 * align256(L.words1);
-    L.off_part = align256(L.sub);
+    L.off_part = 0;
     L.off_grad = L.off_part + align256(L.part);
     L.off_w = L.off_grad + align256(L.grad);
     L.off_lam = L.off_w + align256(L.w);
     L.off_g = L.off_lam + align256(L.lam);
-    L.off_words = L.off_g + align256(L.g);
+    L.off_sub = L.off_g + align256(L.g);
+    L.off_words = L.off_sub + L.sub;
     L.need = L.off_words + L.words;
     return L;
 }
 
-// Whether abp_backward hands the Philox blocks from level 1 to the reverse sweep:
-// the paired kernels and both buffers within the budget -- ABP_ADJ_HANDOFF_BYTES if set (0: never), else half the free device
-// memory not already held by the scratch.
-bool use_handoff(const abp_ctx *ctx) {
+// Bytes abp_backward may take for the Philox blocks that level 1 hands to the reverse sweep
+// (no hand-off where one segment's buffers do not fit): none unless the kernels are the
+// paired ones; ABP_ADJ_HANDOFF_BYTES if set (0: never); else half the free device memory
+// not already held by the scratch.
+double handoff_budget(const abp_ctx *ctx) {
     // both kernels must map blocks and threads to trajectories alike
-    if (!ABP_ADJ_L1_PAIRS || !ABP_ADJ_REV_PAIRS || kL1Threads != kRevPairThreads) return false;
-    const size_t bytes = adj_layout(ctx, true).words;
+    if (!ABP_ADJ_L1_PAIRS || !ABP_ADJ_REV_PAIRS || kL1Threads != kRevPairThreads) return -1.0;
     const char *env = getenv("ABP_ADJ_HANDOFF_BYTES");
-    if (env && *env) return (double)bytes <= strtod(env, nullptr);
+    if (env && *env) return strtod(env, nullptr);
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return -1.0;
     }
-    return bytes <= (free_b + ctx->d_adj.cap) / 2;
+    return (double)((free_b + ctx->d_adj.cap) / 2);
+}
+
+// Segments per launch: as many as this many bytes of buffers hold (one where a segment's
+// own buffers are larger), shared evenly over the launches.  A launch and its events cost
+// the host some 5 us and the device the start and the drain of its blocks, and level 1 of
+// several segments runs side by side: with short segments of small batches that is most
+// of the time.  Backward, one segment per launch against 128 MB: 19,684 trajectories x
+// 3,029 steps, K = 64, 894 -> 647 us; 8,000 x 2,000, K = 64, 497 -> 327; 256 x 4,000,
+// K = 64, 855 -> 479; 8,000 x 2,000, K = 333, 320 -> 303.  64 MB: 694, 426, 484, 313;
+// 256 MB: 625, 321, 477, 308.  A segment of 262,144 trajectories and K = 333 to 1,000 fills
+// the GPU and the buffers by itself.
+#ifndef ABP_ADJ_LAUNCH_BYTES
+#define ABP_ADJ_LAUNCH_BYTES (128 << 20)
+#endif
+int64_t segments_per_launch(const abp_ctx *ctx, bool words, double budget, int64_t n_seg) {
+    const AdjLayout L = adj_layout(ctx, words);
+    int64_t per = (int64_t)((size_t)ABP_ADJ_LAUNCH_BYTES / std::max<size_t>(L.sub + L.words, 1));
+    if (words) per = std::min(per, (int64_t)(budget / (double)std::max<size_t>(L.words, 1)));
+    per = std::max<int64_t>(1, std::min({per, n_seg, (int64_t)65535}));
+    const int64_t launches = (n_seg + per - 1) / per;
+    return launches > 0 ? (n_seg + launches - 1) / launches : 1;
 }
 
 }  // namespace
@@ -942,12 +984,21 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     if (!ctx->ckpt_complete)
         return set_err(ctx, ABP_ESTATE, "abp_backward after abp_load: the checkpoints do not cover the run from step 0");
     const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
-    bool words = use_handoff(ctx);
-    AdjLayout L = adj_layout(ctx, words);
+    const double budget = handoff_budget(ctx);
+    bool words = (double)adj_layout(ctx, true).words <= budget;
+    const int64_t Kc = ctx->cfg.checkpoint_every, n_seg = (ctx->max_steps + Kc - 1) / Kc;
+    int64_t per = segments_per_launch(ctx, words, budget, n_seg);
+    AdjLayout L = adj_layout(ctx, words, per);
     DevBuf &sc = ctx->d_adj;
     if (!sc.p || sc.cap < L.need) {
         sc.release();
         cudaError_t e = cudaMalloc(&sc.p, L.need);
+        if (e != cudaSuccess && per > 1) {  // no room for several segments: one per launch
+            cudaGetLastError();
+            per = 1;
+            L = adj_layout(ctx, words);
+            e = cudaMalloc(&sc.p, L.need);
+        }
         if (e != cudaSuccess && words) {  // no room for the hand-off: draw the blocks twice instead
             cudaGetLastError();
             words = false;
@@ -963,7 +1014,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     }
     sc.bytes = L.need;
     char *base = (char *)sc.p;
-    float4 *sub[2] = {(float4 *)base, (float4 *)(base + align256(L.sub1))};
+    float4 *sub[2] = {(float4 *)(base + L.off_sub), (float4 *)(base + L.off_sub + align256(L.sub1))};
     uint4 *wbuf[2] = {(uint4 *)(base + L.off_words), (uint4 *)(base + L.off_words + align256(L.words1))};
     double *partials = (double *)(base + L.off_part);
     double *gdev = (double *)(base + L.off_grad);
@@ -995,6 +1046,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         a.nz = ctx->noise();
         a.sub = sub[0];
         a.n_sub = n_sub;
+        a.per = (int)per;
         a.words = nullptr;
         a.tile0 = 0;
         a.n_blk = n_sub * (kSub / 4);
@@ -1007,8 +1059,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         e = cudaMemsetAsync(sv.lam, 0, lam_bytes, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(sv.G, 0, g_bytes, s);
         if (e != cudaSuccess) return set_err(ctx, ABP_ECUDA, "abp_backward: clear", e);
-        const int64_t Kc = ctx->cfg.checkpoint_every;
-        const int64_t n_seg = (ctx->max_steps + Kc - 1) / Kc;
+        const int64_t n_run = (n_seg + per - 1) / per;  // launches of each kernel
         // blocks per tile: tiles hold up to kThreads * ppt trajectories
         const int cap = kThreads * std::max(ctx->ppt, 1);
         const int sub1 = ABP_ADJ_L1_PAIRS ? pair_blocks_per_tile(ctx, kL1Threads) : (cap + kL1Threads - 1) / kL1Threads;
@@ -1035,7 +1086,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         }
         struct Group {
             cudaStream_t rev, l1;
-            cudaEvent_t *l1_done, *rev_done;  // [2] by segment parity
+            cudaEvent_t *l1_done, *rev_done;  // [2] by launch parity
             int t0, t1;
         } grp[kAdjGroups];
         for (int g = 0; g < n_grp; ++g) {
@@ -1053,20 +1104,22 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         auto record = [&](cudaEvent_t ev, cudaStream_t st) {
             if (e == cudaSuccess) e = cudaEventRecord(ev, st);
         };
-        // level 1 of segment j writes buffer j % 2; it may start once the reverse
-        // sweep of segment j + 2, the last reader of that buffer, has finished
+        // launch j covers the segments [j per, (j + 1) per); level 1 of launch j writes
+        // buffer j % 2 and may start once the reverse sweep of launch j + 2, the last
+        // reader of that buffer, has finished
+        auto segments = [&](int64_t j) { return (unsigned)std::min(per, n_seg - j * per); };
         auto level1 = [&](const Group &g, int64_t j) {
             AdjArgs aj = a;
             aj.sub = sub[j & 1];
             aj.tile0 = g.t0;
-            const unsigned g1 = (unsigned)((int64_t)(g.t1 - g.t0) * sub1);
+            const dim3 g1((unsigned)((int64_t)(g.t1 - g.t0) * sub1), segments(j));
             if (words) {
                 aj.words = wbuf[j & 1];
-                adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
+                adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
             } else if (ABP_ADJ_L1_PAIRS)
-                adjoint_level1_pair_kernel<false><<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
+                adjoint_level1_pair_kernel<false><<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
             else
-                adjoint_level1_kernel<<<g1, kL1Threads, 0, g.l1>>>(aj, j, sub1);
+                adjoint_level1_kernel<<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
             record(g.l1_done[j & 1], g.l1);
         };
         auto reverse = [&](const Group &g, int64_t j) {
@@ -1077,11 +1130,11 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             const unsigned g2 = (unsigned)((int64_t)(g.t1 - g.t0) * sub2);
             if (words) {
                 as.words = wbuf[j & 1];
-                adjoint_reverse_pair_kernel<true><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j, sub2, window);
+                adjoint_reverse_pair_kernel<true><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
             } else if (ABP_ADJ_REV_PAIRS)
-                adjoint_reverse_pair_kernel<false><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j, sub2, window);
+                adjoint_reverse_pair_kernel<false><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
             else
-                adjoint_reverse_kernel<<<g2, kRevThreads, 0, g.rev>>>(as, sv, j, sub2, window);
+                adjoint_reverse_kernel<<<g2, kRevThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
             record(g.rev_done[j & 1], g.rev);
             ctx->launches += 2;
         };
@@ -1089,15 +1142,15 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         for (int g = 0; g < n_grp; ++g) {
             wait(grp[g].l1, start);
             if (g > 0) wait(grp[g].rev, start);
-            if (n_seg > 0) level1(grp[g], n_seg - 1);
+            if (n_run > 0) level1(grp[g], n_run - 1);
         }
-        for (int64_t seg = n_seg - 1; e == cudaSuccess && seg >= 0; --seg)
+        for (int64_t j = n_run - 1; e == cudaSuccess && j >= 0; --j)
             for (int g = 0; g < n_grp; ++g) {
-                if (seg > 0) {
-                    if (seg + 1 < n_seg) wait(grp[g].l1, grp[g].rev_done[(seg + 1) & 1]);
-                    level1(grp[g], seg - 1);
+                if (j > 0) {
+                    if (j + 1 < n_run) wait(grp[g].l1, grp[g].rev_done[(j + 1) & 1]);
+                    level1(grp[g], j - 1);
                 }
-                reverse(grp[g], seg);
+                reverse(grp[g], j);
             }
         for (int g = 1; g < n_grp; ++g) {  // also after an error: the caller's stream then follows all launches
             cudaEventRecord(end, grp[g].rev);
