@@ -244,12 +244,16 @@ ABP_API abp_status abp_load(abp_ctx *ctx, const void *buf, size_t bytes);
  * Requires a completed abp_integrate with checkpoint_every > 0 (otherwise
  * ABP_ESTATE); recomputes each checkpoint interval forward and sweeps it in
  * reverse, accumulating in FP64.  Device scratch (context-owned, kept for the
- * next call): 32 bytes per trajectory per 8 steps of checkpoint_every plus 64
- * bytes per trajectory; when checkpoint_every is a multiple of 8, also 8 bytes
- * per trajectory per step of checkpoint_every for handing the noise of each
- * interval's first re-run to its reverse sweep, if that fits in the budget the
- * environment variable ABP_ADJ_HANDOFF_BYTES gives (0: never), by default half
- * the free device memory -- else the noise is drawn again.  The results are the
+ * next call): 64 bytes per trajectory; 32 bytes per trajectory per 8 steps of
+ * checkpoint_every; 8 bytes per trajectory per step of checkpoint_every for
+ * handing the noise of each interval's first re-run to its reverse sweep, if that
+ * fits in the budget the environment variable ABP_ADJ_HANDOFF_BYTES gives (0:
+ * never), by default half the free device memory -- else the noise is drawn
+ * again; short intervals are taken several at a time, up to 128 MB in all.
+ * Batches of at most 32,768 trajectories take 32 bytes per trajectory per step
+ * instead, for as many intervals as 512 MB hold (ABP_ADJ_STATE_BYTES; 0: never),
+ * within the same budget.  Where an allocation fails the smaller forms are used
+ * (one interval at a time, then the noise drawn again).  The results are the
  * same bit for bit either way. */
 ABP_API abp_status abp_backward(abp_ctx *ctx, const double *dJ_dmean_v, double *grad);
 

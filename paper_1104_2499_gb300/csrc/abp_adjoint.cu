@@ -733,7 +733,9 @@ __global__ void __launch_bounds__(kRevThreads, ABP_ADJ_MIN_BLOCKS) adjoint_rever
 
 // The reverse kernel with two trajectories per thread (trajectories li and
 // li + blockDim.x of the block's 2 blockDim.x), `sub` blocks per tile.
-template <bool WORDS>
+// MULTI: the launch covers n segments (without it the loop below costs the kernel at its
+// register cap a spill, 1% of the sweep).
+template <bool WORDS, bool MULTI>
 __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) adjoint_reverse_pair_kernel(AdjArgs a, SegView sv, int64_t seg0,
                                                                                int n, int sub, int64_t window) {
     __shared__ WordStage stage[WORDS ? kStages : 1];
@@ -754,7 +756,7 @@ __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) 
                             dchk(b.tile_first[tile] + (second ? li + (int)blockDim.x : li), T, b.dbg)};
     const StepStream ss[2] = {step_stream((uint64_t)idx[0] + a.nz.traj_base, a.K),
                               step_stream((uint64_t)idx[1] + a.nz.traj_base, a.K)};
-    for (int i = n - 1; i >= 0; --i) {
+    for (int i = MULTI ? n - 1 : 0; i >= 0; --i) {
         const int64_t seg = seg0 + i, s0 = seg * K;
         if (s0 >= N) continue;
         float4 l0 = sv.lam[idx[0]], l1 = sv.lam[idx[1]];
@@ -774,6 +776,143 @@ __global__ void __launch_bounds__(kRevPairThreads, ABP_ADJ_REV_PAIR_MIN_BLOCKS) 
             for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx[1]] += (double)acc[q].y;
         }
     }
+}
+
+// Small batches: level 1 leaves every step's state, (force phase, v, e, sigma z) in one
+// 16-byte row, and the sweep only reads them.  There a warp has its scheduler to itself
+// and a launch's time is the length of one trajectory's sweep: the pair kernel's thread
+// re-runs and sweeps two trajectories, some 62 instructions a step, the one here sweeps
+// one, about 26, while level 1 runs all segments of the launch side by side.
+__global__ void __launch_bounds__(kL1Threads) adjoint_states_kernel(AdjArgs a, int64_t seg0, int sub) {
+    const Batch &b = a.b;
+    const int64_t seg = seg0 + blockIdx.y;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
+    const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
+    const int set = b.tile_set[tile];
+    const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
+    const int64_t s0 = seg * K;
+    if (s0 >= N) return;  // uniform over the block
+    const int64_t s1 = min(s0 + K, N);
+    const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, a.nz.dt);  // the forward's own coefficients
+    if (li >= b.tile_count[tile]) return;
+    const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
+    const StepStream ss = step_stream((uint64_t)idx + a.nz.traj_base, a.K);
+    const float4 c0 = a.ck.ck[(size_t)dchk(seg, a.ck.n_slots, b.dbg) * T + idx];
+    float y = c0.x, yacc = c0.y, v = c0.z, e = c0.w;
+    float pb = phase_base(y);
+    float4 *const rows = segment_slots(a, (int)blockIdx.y) + idx;  // K rows per segment
+    int64_t n = s0;
+    auto row = [&](int64_t m, float sz) {
+        rows[(size_t)dchk(m - s0, a.n_sub, b.dbg) * T] = make_float4(phase_arg(pb, yacc), v, e, sz);
+    };
+    while (n < s1) {
+        float nrs[4], tr[4];
+        block_noise(k, ss, a.K, (uint32_t)(n >> 2), nrs, tr);
+        if ((n & 3) == 0 && n + 4 <= s1) {  // no fold falls inside a block of four steps
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                row(n + i, nrs[i] * tr[i]);
+                em_step_f32(k, nrs[i], tr[i], pb, yacc, v, e);
+            }
+            n += 4;
+            if ((n & (kBlockSteps - 1)) == 0) fold(y, yacc, pb);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (i == (int)(n & 3) && n < s1) {
+                    row(n, nrs[i] * tr[i]);
+                    fwd(k, nrs[i], tr[i], n, y, yacc, pb, v, e);
+                    ++n;
+                }
+        }
+    }
+}
+
+// The sweep over the rows of a launch's n segments, one trajectory per thread in blocks of
+// one warp.  The rows of consecutive segments follow one another, so the copies into the
+// thread's own ring (cp.async, kRowGroups - 1 groups of kRowGroup rows ahead, no barrier:
+// a thread reads only what it copied) run on across segments.
+constexpr int kRowGroup = 8, kRowGroups = 8, kSweepThreads = 32;
+
+__global__ void __launch_bounds__(kSweepThreads) adjoint_sweep_kernel(AdjArgs a, SegView sv, int64_t seg0, int n,
+                                                                      int sub, int64_t window) {
+    __shared__ float4 ring[kRowGroup * kRowGroups][kSweepThreads];
+    const Batch &b = a.b;
+    const int tile = a.tile0 + (int)blockIdx.x / sub;
+    const int li = ((int)blockIdx.x % sub) * kSweepThreads + (int)threadIdx.x;
+    const int set = b.tile_set[tile];
+    const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
+    const int64_t first = seg0 * K;
+    if (first >= N) return;  // uniform over the block
+    if (li >= b.tile_count[tile]) return;
+    const abp_params p = b.params[set];
+    const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, a.nz.dt);  // the forward's own coefficients
+    const float dtf = (float)a.nz.dt;
+    const float kx = (float)(-2.0 * kPi / p.L);
+    const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
+    const int rows = (int)(min(first + n * K, N) - first);
+    const float4 *const src = a.sub + idx;
+    auto fetch = [&](int g) {
+        if (g >= 0)
+#pragma unroll
+            for (int i = 0; i < kRowGroup; ++i) {
+                const int r = g * kRowGroup + i;
+                if (r < rows)
+                    cp_async16(&ring[(g % kRowGroups) * kRowGroup + i][threadIdx.x],
+                               src + (size_t)dchk((int64_t)r, a.n_sub * a.per, b.dbg) * T);
+            }
+        cp_async_commit();
+    };
+    const int top = (rows - 1) / kRowGroup;
+#pragma unroll 1
+    for (int i = 0; i < kRowGroups - 1; ++i) fetch(top - i);
+    float4 l0 = sv.lam[idx];
+    float lx = l0.x, lv = l0.y, le = l0.z;
+    float acc[6] = {0, 0, 0, 0, 0, 0};
+    double G[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) G[q] = sv.G[(size_t)q * T + idx];
+    int seg = (int)((rows - 1) / K);   // the segment of the launch being swept
+    int begin = (int)(seg * K);        // its first row
+    auto enter = [&]() {               // windowed adjoint: the window ending at step (seg0 + seg + 1) K starts from zero
+        if (window > 0 && ((seg0 + seg + 1) * K) % window == 0) lx = lv = le = 0.0f;
+    };
+    auto leave = [&]() {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            G[q] += (double)acc[q];
+            acc[q] = 0.0f;
+        }
+        --seg;
+        begin -= (int)K;
+        if (seg >= 0) enter();
+    };
+    enter();
+    for (int g = top; g >= 0; --g) {
+        fetch(g - (kRowGroups - 1));
+        cp_async_wait<kRowGroups - 1>();  // this thread's copies of group g have landed
+        const int r0 = g * kRowGroup;
+        const float4(*const rg)[kSweepThreads] = ring + (g % kRowGroups) * kRowGroup;
+        if (r0 >= begin && r0 + kRowGroup <= rows) {
+#pragma unroll
+            for (int i = kRowGroup - 1; i >= 0; --i) {
+                const float4 c = rg[i][threadIdx.x];
+                reverse_step(k, kx, dtf, c.x, c.y, c.z, c.w, lx, lv, le, acc);
+            }
+            if (r0 == begin) leave();
+        } else {
+#pragma unroll 1
+            for (int i = kRowGroup - 1; i >= 0; --i) {
+                if (r0 + i >= rows) continue;
+                const float4 c = rg[i][threadIdx.x];
+                reverse_step(k, kx, dtf, c.x, c.y, c.z, c.w, lx, lv, le, acc);
+                if (r0 + i == begin) leave();
+            }
+        }
+    }
+    sv.lam[idx] = make_float4(lx, lv, le, 0.0f);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx] = G[q];
 }
 
 // Per tile: the initial-condition term, the parameter scales and the caller's
@@ -897,10 +1036,10 @@ int pair_blocks_per_tile(const abp_ctx *ctx, int threads) {
     return (cap + 2 * threads - 1) / (2 * threads);
 }
 
-AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1) {
+AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool states = false) {
     AdjLayout L;
     const int64_t T = ctx->total_traj, Kc = ctx->cfg.checkpoint_every;
-    const int64_t n_sub = sub_slots(Kc);
+    const int64_t n_sub = states ? Kc : sub_slots(Kc);
     L.sub1 = sizeof(float4) * (size_t)(per * n_sub) * (size_t)T;
     L.sub = 2 * align256(L.sub1);  // two buffers, alternating by launch
     L.part = sizeof(double) * 6 * (size_t)std::max(ctx->n_tiles, 1);
@@ -939,6 +1078,28 @@ double handoff_budget(const abp_ctx *ctx) {
     return (double)((free_b + ctx->d_adj.cap) / 2);
 }
 
+// Whether level 1 hands every step's state to the sweep (adjoint_states_kernel): batches of
+// at most kStateTraj trajectories whose segments fit ABP_ADJ_STATE_BYTES (0: never) and
+// the hand-off's budget.  Backward of the pair kernels against this: 256 trajectories x
+// 4,000 steps, K = 64, 482 -> 267 us; 8,000 x 2,000, K = 64, 333 -> 206, K = 333, 309 ->
+// 210; 8,192 x 4,000, K = 1,000, 487 -> 319; 16,384 x 4,000, K = 200, 869 -> 478; 32,768 x
+// 2,000, K = 64, 588 -> 505, K = 500, 526 -> 485: beyond that the SMs hold more warps than
+// the ring leaves room for and the rows' 32 bytes a step come from HBM.  Fewer bytes mean
+// more launches (128 MB: 249, 240 and 488 us for the second to fourth of these, 256 MB:
+// 217, 212 and 369).
+#ifndef ABP_ADJ_STATE_TRAJ
+#define ABP_ADJ_STATE_TRAJ 32768
+#endif
+constexpr int64_t kStateTraj = ABP_ADJ_STATE_TRAJ;
+double state_bytes() {
+    const char *env = getenv("ABP_ADJ_STATE_BYTES");
+    return env && *env ? std::min(strtod(env, nullptr), 4e9) : 512.0 * (1 << 20);  // row numbers stay in 32 bits
+}
+bool use_states(const abp_ctx *ctx, double budget) {
+    return ctx->total_traj <= kStateTraj &&
+           (double)adj_layout(ctx, false, 1, true).sub <= std::min(budget, state_bytes());
+}
+
 // Segments per launch: as many as this many bytes of buffers hold (one where a segment's
 // own buffers are larger), shared evenly over the launches.  A launch and its events cost
 // the host some 5 us and the device the start and the drain of its blocks, and level 1 of
@@ -951,10 +1112,12 @@ double handoff_budget(const abp_ctx *ctx) {
 #ifndef ABP_ADJ_LAUNCH_BYTES
 #define ABP_ADJ_LAUNCH_BYTES (128 << 20)
 #endif
-int64_t segments_per_launch(const abp_ctx *ctx, bool words, double budget, int64_t n_seg) {
-    const AdjLayout L = adj_layout(ctx, words);
-    int64_t per = (int64_t)((size_t)ABP_ADJ_LAUNCH_BYTES / std::max<size_t>(L.sub + L.words, 1));
+int64_t segments_per_launch(const abp_ctx *ctx, bool words, bool states, double budget, int64_t n_seg) {
+    const AdjLayout L = adj_layout(ctx, words, 1, states);
+    int64_t per = (int64_t)((states ? state_bytes() : (double)ABP_ADJ_LAUNCH_BYTES) /
+                            (double)std::max<size_t>(L.sub + L.words, 1));
     if (words) per = std::min(per, (int64_t)(budget / (double)std::max<size_t>(L.words, 1)));
+    if (states) per = std::min(per, (int64_t)(budget / (double)std::max<size_t>(L.sub, 1)));
     per = std::max<int64_t>(1, std::min({per, n_seg, (int64_t)65535}));
     const int64_t launches = (n_seg + per - 1) / per;
     return launches > 0 ? (n_seg + launches - 1) / launches : 1;
@@ -985,17 +1148,19 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         return set_err(ctx, ABP_ESTATE, "abp_backward after abp_load: the checkpoints do not cover the run from step 0");
     const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
     const double budget = handoff_budget(ctx);
-    bool words = (double)adj_layout(ctx, true).words <= budget;
+    bool states = use_states(ctx, budget);
+    bool words = !states && (double)adj_layout(ctx, true).words <= budget;
     const int64_t Kc = ctx->cfg.checkpoint_every, n_seg = (ctx->max_steps + Kc - 1) / Kc;
-    int64_t per = segments_per_launch(ctx, words, budget, n_seg);
-    AdjLayout L = adj_layout(ctx, words, per);
+    int64_t per = segments_per_launch(ctx, words, states, budget, n_seg);
+    AdjLayout L = adj_layout(ctx, words, per, states);
     DevBuf &sc = ctx->d_adj;
     if (!sc.p || sc.cap < L.need) {
         sc.release();
         cudaError_t e = cudaMalloc(&sc.p, L.need);
-        if (e != cudaSuccess && per > 1) {  // no room for several segments: one per launch
+        if (e != cudaSuccess && (per > 1 || states)) {  // no room for several segments: one per launch
             cudaGetLastError();
             per = 1;
+            states = false;
             L = adj_layout(ctx, words);
             e = cudaMalloc(&sc.p, L.need);
         }
@@ -1045,7 +1210,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         a.ck = ctx->ckpt();
         a.nz = ctx->noise();
         a.sub = sub[0];
-        a.n_sub = n_sub;
+        a.n_sub = states ? Kc : n_sub;
         a.per = (int)per;
         a.words = nullptr;
         a.tile0 = 0;
@@ -1065,6 +1230,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         const int sub1 = ABP_ADJ_L1_PAIRS ? pair_blocks_per_tile(ctx, kL1Threads) : (cap + kL1Threads - 1) / kL1Threads;
         const int sub2 = ABP_ADJ_REV_PAIRS ? pair_blocks_per_tile(ctx, kRevPairThreads)
                                            : (cap + kRevThreads - 1) / kRevThreads;
+        const int sub_st = (cap + kL1Threads - 1) / kL1Threads, sub_sw = (cap + kSweepThreads - 1) / kSweepThreads;
         // The tiles in two halves, each with its own pair of streams: a trajectory's sweep
         // depends on no other's, so while one half's launch of a segment drains (its last
         // blocks fill the SMs partly, and its next launch waits for them) the other half's
@@ -1073,7 +1239,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         // 131,072 3.09 -> 2.71, 1,048,576 2.40 -> 2.38 (three, four and six groups: within 2%
         // of two).  A batch with fewer blocks than SMs runs in one group: it leaves SMs
         // free anyway, and each launch costs host time.
-        const int n_grp = ctx->n_tiles >= 2 && (int64_t)ctx->n_tiles * sub2 >= ctx->sm_count ? kAdjGroups : 1;
+        const int n_grp = !states && ctx->n_tiles >= 2 && (int64_t)ctx->n_tiles * sub2 >= ctx->sm_count ? kAdjGroups : 1;
         if (!ctx->adj_stream[0]) {
             for (int i = 0; e == cudaSuccess && i < 2 * kAdjGroups - 1; ++i)
                 e = cudaStreamCreateWithFlags(&ctx->adj_stream[i], cudaStreamNonBlocking);
@@ -1113,7 +1279,10 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             aj.sub = sub[j & 1];
             aj.tile0 = g.t0;
             const dim3 g1((unsigned)((int64_t)(g.t1 - g.t0) * sub1), segments(j));
-            if (words) {
+            if (states)
+                adjoint_states_kernel<<<dim3((unsigned)((g.t1 - g.t0) * sub_st), segments(j)), kL1Threads, 0, g.l1>>>(
+                    aj, j * per, sub_st);
+            else if (words) {
                 aj.words = wbuf[j & 1];
                 adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
             } else if (ABP_ADJ_L1_PAIRS)
@@ -1128,12 +1297,16 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             as.sub = sub[j & 1];
             as.tile0 = g.t0;
             const unsigned g2 = (unsigned)((int64_t)(g.t1 - g.t0) * sub2);
-            if (words) {
-                as.words = wbuf[j & 1];
-                adjoint_reverse_pair_kernel<true><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
-            } else if (ABP_ADJ_REV_PAIRS)
-                adjoint_reverse_pair_kernel<false><<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
-            else
+            if (states) {
+                adjoint_sweep_kernel<<<(unsigned)((g.t1 - g.t0) * sub_sw), kSweepThreads, 0, g.rev>>>(
+                    as, sv, j * per, (int)segments(j), sub_sw, window);
+            } else if (ABP_ADJ_REV_PAIRS) {
+                if (words) as.words = wbuf[j & 1];
+                const auto kernel =
+                    words ? (per > 1 ? adjoint_reverse_pair_kernel<true, true> : adjoint_reverse_pair_kernel<true, false>)
+                          : (per > 1 ? adjoint_reverse_pair_kernel<false, true> : adjoint_reverse_pair_kernel<false, false>);
+                kernel<<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
+            } else
                 adjoint_reverse_kernel<<<g2, kRevThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
             record(g.rev_done[j & 1], g.rev);
             ctx->launches += 2;

@@ -51,9 +51,10 @@ abp_status cuda_fail(abp_ctx *ctx, cudaError_t e, const char *what) {
 // Resident blocks per SM of the work queue for a batch of n_tiles tiles: the
 // kernel's occupancy, but no more blocks than leave 1.5 tiles to each.  An item
 // waits for its tile's previous round; with about one tile per block the blocks
-// of a round outrun the tiles and idle on those waits (load sweep, 512 tiles:
-// 9.95e11 particle-steps/s on 304 blocks, 9.64e11 on 456).  One block already
-// draws an SM's full rate, so fewer blocks cost little elsewhere.
+// of a round outrun the tiles and idle on those waits (load sweep, 512 tiles, items of
+// 1,000 steps: 1.073e12 particle-steps/s on 304 blocks, 9.80e11 on 456; of 10^4 steps
+// 1.062e12 and 8.67e11).  One block already draws an SM's full rate, so fewer blocks
+// cost little elsewhere.
 int wq_blocks_per_sm(int bps, int64_t n_tiles, int sms) {
     const int64_t fit = (2 * n_tiles) / (3 * (int64_t)std::max(sms, 1));
     return (int)std::max<int64_t>(1, std::min<int64_t>(std::max(bps, 1), fit));

@@ -490,10 +490,10 @@ static_assert(kWsSlotSteps == kBlockSteps, "a slot ends where a fold does");
 constexpr int kWsProducers = 3;
 // Narrow launches planned at most this wide run warp-specialised, as 32-thread
 // stepping blocks.  Measured on the work-items sweep (one-trajectory sets, 10^4
-// steps per cycle): 2^14 items, planned 64 wide (256 blocks), 0.42 ms per cycle
-// on the plain narrow kernel and 0.34 ms warp-specialised (512 blocks of four
-// warps, all resident); at 2^15 (128 wide) the warp-specialised grid would no
-// longer fit on the SMs at once.
+// steps per cycle): 2^14 items, planned 64 wide (256 blocks), 0.30 ms per cycle on
+// the plain narrow kernel and as much warp-specialised (512 blocks of four warps, all
+// resident); a set of 4,096 trajectories, 32 wide, 0.31 and 0.16 ms; at 2^15 (128 wide)
+// the warp-specialised grid would no longer fit on the SMs at once.
 #ifndef ABP_WS_WIDEST
 #define ABP_WS_WIDEST 64
 #endif

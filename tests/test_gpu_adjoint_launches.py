@@ -1,5 +1,6 @@
 """Adjoint launches that cover several segments: level 1 with a segment per grid row, the reverse
-sweep over the launch's segments, with the bits of one segment per launch."""
+sweep over the launch's segments, with the bits of one segment per launch; and the small batches'
+form, in which level 1 leaves every step's state for the sweep."""
 import numpy as np
 import pytest
 
@@ -8,6 +9,7 @@ from paper_1104_2499_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
+STATES = 2 * 16 * 366  # both buffers of one step: a 16-byte row per trajectory
 SEGMENT = 2 * 16 * 6 * 2 * 2 * 128  # both hand-off buffers of one segment: 6 blocks of 128, K = 8 or 5
 
 
@@ -36,13 +38,19 @@ def grads(abp, K, window):
 @pytest.mark.parametrize("window", [0, 40])
 def test_segments_per_launch(abp, monkeypatch, K, slots, window):
     out = {}
+    monkeypatch.setenv("ABP_ADJ_STATE_BYTES", "0")
     for n in (1, 3, 5, None):
         monkeypatch.setenv("ABP_ADJ_HANDOFF_BYTES", "" if n is None else str(n * slots * SEGMENT))
         out[n] = grads(abp, K, window)
     monkeypatch.setenv("ABP_ADJ_HANDOFF_BYTES", "0")
     out[0] = grads(abp, K, window)
+    monkeypatch.delenv("ABP_ADJ_HANDOFF_BYTES")
+    states = {}
+    for n in (1, 3, 5, None):  # a buffer is rounded up to 256 bytes
+        monkeypatch.setenv("ABP_ADJ_STATE_BYTES", "" if n is None else str(n * (K * STATES + 512)))
+        states[n] = grads(abp, K, window)
     n_seg = -(-203 // K)
-    for n, (launches, g, t) in out.items():
+    for n, (launches, g, t) in [*out.items(), *states.items()]:
         runs = -(-n_seg // n) if n else 1
         assert launches == 2 * runs + 2  # level 1 and reverse per run, the tile and the set sums
         np.testing.assert_array_equal(g, out[1][1])
