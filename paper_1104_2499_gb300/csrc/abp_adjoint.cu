@@ -29,21 +29,11 @@ namespace {
 #ifndef ABP_ADJ_SUB
 #define ABP_ADJ_SUB 8
 #endif
-#ifndef ABP_ADJ_MIN_BLOCKS
-#define ABP_ADJ_MIN_BLOCKS 2
-#endif
-#ifndef ABP_ADJ_REV_THREADS
-#define ABP_ADJ_REV_THREADS 256
-#endif
-// Reverse sweep with two trajectories per thread in paired FP32 (1) or one (0),
-// and the block size and minimum resident blocks of the paired reverse kernel.
+// Block size and minimum resident blocks of the paired reverse kernel.
 // Measured on the full differentiation workload (1M x 1e5, K = 1,000),
 // backward time: one trajectory per thread 318 ms; paired, 210 registers (two
 // 128-thread blocks per SM) 313 ms; paired, capped at 168 registers for three
 // blocks per SM (no spills) 304 ms; paired with 4-step sub-chunks 324 ms.
-#ifndef ABP_ADJ_REV_PAIRS
-#define ABP_ADJ_REV_PAIRS 1
-#endif
 #ifndef ABP_ADJ_REV_PAIR_THREADS
 #define ABP_ADJ_REV_PAIR_THREADS 128
 #endif
@@ -51,17 +41,11 @@ namespace {
 #define ABP_ADJ_REV_PAIR_MIN_BLOCKS 3
 #endif
 constexpr int kRevPairThreads = ABP_ADJ_REV_PAIR_THREADS;
-// Level 1 with two trajectories per thread in paired FP32 (1) or one (0).
-#ifndef ABP_ADJ_L1_PAIRS
-#define ABP_ADJ_L1_PAIRS 1
-#endif
 // Aligned whole chunks of the paired level 1 stepped in groups of this many per
 // loop iteration (1: one chunk per iteration).
 #ifndef ABP_ADJ_L1_GROUP
 #define ABP_ADJ_L1_GROUP 4
 #endif
-// Threads per block of the register-heavy reverse kernel (a multiple of 32).
-constexpr int kRevThreads = ABP_ADJ_REV_THREADS;
 // Threads per block of the level-1 kernel: small blocks, so that one fits on
 // an SM beside the reverse kernel's blocks and fills the issue slots they
 // leave idle.
@@ -83,7 +67,6 @@ struct SegChunks {
     __device__ __forceinline__ SegChunks(int64_t a, int64_t b) : s0(a), s1(b), c0(a / kSub), n((int)((b + kSub - 1) / kSub - a / kSub)) {}
     __device__ __forceinline__ int64_t begin(int j) const { return j == 0 ? s0 : (c0 + j) * kSub; }
     __device__ __forceinline__ int64_t end(int j) const { return j == n - 1 ? s1 : (c0 + j + 1) * kSub; }
-    __device__ __forceinline__ bool whole(int j) const { return end(j) - begin(j) == kSub; }
     // chunks [first_whole, last_whole) are whole
     __device__ __forceinline__ int first_whole() const { return s0 % kSub ? 1 : 0; }
     __device__ __forceinline__ int last_whole() const { return max(s1 % kSub ? n - 1 : n, first_whole()); }
@@ -233,43 +216,9 @@ __device__ __forceinline__ void block_sum6(double (&a)[6], double (*red)[6]) {
     }
 }
 
-// Level 1 of segment [s0, s1) of one trajectory: re-run from its checkpoint
-// (y, yacc, v, e) = c0, leaving the state at the start of each chunk in the
-// sub-checkpoint scratch.  Whole chunks take their noise one Philox block per four
-// steps (the forward's own path); partial ones step one at a time.
-__device__ __forceinline__ void level1_segment(const AdjArgs &a, float4 *slots, const Coef<float> &k, const StepStream &ss,
-                                               int64_t idx, int64_t s0, int64_t s1, float4 c0) {
-    const int64_t T = a.b.total_traj;
-    const SegChunks seg(s0, s1);
-    float y = c0.x, yacc = c0.y, v = c0.z, e = c0.w;
-    float pb = phase_base(y);
-    NoiseCursor nc;
-    nc.valid = false;
-    nc.m = 0;
-    for (int j = 0; j < seg.n; ++j) {
-        const int64_t n0 = seg.begin(j);
-        slots[(size_t)dchk(j, a.n_sub, a.b.dbg) * T + idx] = make_float4(y, yacc, v, e);
-        if (seg.whole(j)) {
-#pragma unroll
-            for (int b2 = 0; b2 < kSub / 4; ++b2) {
-                float nrs[4], tr[4];
-                block_noise(k, ss, a.K, (uint32_t)(n0 >> 2) + b2, nrs, tr);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) em_step_f32(k, nrs[i], tr[i], pb, yacc, v, e);
-            }
-            if (((n0 + kSub) & (kBlockSteps - 1)) == 0) fold(y, yacc, pb);
-        } else {
-            const int len = (int)(seg.end(j) - n0);
-            for (int i = 0; i < len; ++i) {
-                float nrs, tr;
-                nc.at(k, ss, a.K, n0 + i, nrs, tr);
-                fwd(k, nrs, tr, n0 + i, y, yacc, pb, v, e);
-            }
-        }
-    }
-}
-
-// level1_segment for two trajectories (idx0, idx1) of one thread: whole
+// Level 1 of segment [s0, s1) of two trajectories (idx[0], idx[1]) of one thread: re-run
+// from their checkpoints c0, c1, leaving the state at the start of each chunk in the
+// sub-checkpoint scratch.  Whole
 // chunks step the pair with paired FP32 instructions (same operations
 // as em_step_f32 / box_muller_f32 on each half, so the sub-checkpoints are the
 // scalar ones bit for bit); other chunks step each trajectory on its own.
@@ -376,66 +325,6 @@ __device__ __forceinline__ void level1_segment2(const AdjArgs &a, float4 *slots,
     if (j < seg.n) partial_chunk(j);
 }
 
-// Level 2 and the reverse sweep of segment [s0, s1): its kSub-step chunks in
-// reverse order, each re-run from its sub-checkpoint into registers and swept
-// backwards.  Each chunk's sub-checkpoint is loaded one chunk ahead, so its
-// memory latency overlaps the previous chunk's arithmetic.
-__device__ __forceinline__ void reverse_chunks(const AdjArgs &a, const float4 *slots, const Coef<float> &k,
-                                               const StepStream &ss, float kx, float dtf, int64_t idx, int64_t s0, int64_t s1, float &lx, float &lv,
-                                               float &le, float (&acc)[6]) {
-    const int64_t T = a.b.total_traj;
-    const SegChunks seg(s0, s1);
-    NoiseCursor nc;
-    nc.valid = false;
-    nc.m = 0;
-    float4 c_next = slots[(size_t)dchk(seg.n - 1, a.n_sub, a.b.dbg) * T + idx];
-    for (int j = seg.n - 1; j >= 0; --j) {
-        const int64_t n0 = seg.begin(j);
-        const int len = (int)(seg.end(j) - n0);
-        const float4 cj = c_next;
-        if (j > 0) c_next = slots[(size_t)dchk(j - 1, a.n_sub, a.b.dbg) * T + idx];
-        float y = cj.x, yacc = cj.y, v = cj.z, e = cj.w;
-        float pb = phase_base(y);
-        float ys[kSub], vs[kSub], es[kSub], szs[kSub];  // ys: the force phase of each step
-        if (len == kSub) {
-            // no fold falls inside a whole chunk (folds come after multiples of kBlockSteps)
-#pragma unroll
-            for (int b2 = 0; b2 < kSub / 4; ++b2) {
-                float nrs[4], tr[4];
-                block_noise(k, ss, a.K, (uint32_t)(n0 >> 2) + b2, nrs, tr);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int q = 4 * b2 + i;
-                    ys[q] = phase_arg(pb, yacc);
-                    vs[q] = v;
-                    es[q] = e;
-                    szs[q] = nrs[i] * tr[i];
-                    em_step_f32(k, nrs[i], tr[i], pb, yacc, v, e);
-                }
-            }
-#pragma unroll
-            for (int i = kSub - 1; i >= 0; --i) reverse_step(k, kx, dtf, ys[i], vs[i], es[i], szs[i], lx, lv, le, acc);
-        } else {
-            nc.valid = false;
-#pragma unroll
-            for (int i = 0; i < kSub; ++i) {
-                if (i < len) {
-                    float nrs, tr;
-                    nc.at(k, ss, a.K, n0 + i, nrs, tr);
-                    ys[i] = phase_arg(pb, yacc);
-                    vs[i] = v;
-                    es[i] = e;
-                    szs[i] = nrs * tr;
-                    fwd(k, nrs, tr, n0 + i, y, yacc, pb, v, e);
-                }
-            }
-#pragma unroll
-            for (int i = kSub - 1; i >= 0; --i)
-                if (i < len) reverse_step(k, kx, dtf, ys[i], vs[i], es[i], szs[i], lx, lv, le, acc);
-        }
-    }
-}
-
 // reverse_step of two trajectories in the halves of FP32 pairs, same
 // operations in the same order as the scalar function (each half rounded as
 // the scalar operation), so the gradient sums are the scalar kernel's bits.
@@ -485,7 +374,10 @@ __device__ __forceinline__ void reverse_step_x2(const RevCoef2 &c, float2 ph, fl
     le = nle;
 }
 
-// reverse_chunks for two trajectories of one thread (idx[0], idx[1]): whole
+// Level 2 and the reverse sweep of segment [s0, s1) for two trajectories of one thread
+// (idx[0], idx[1]): its kSub-step chunks in reverse order, each re-run from its
+// sub-checkpoint into registers and swept backwards, each sub-checkpoint loaded one chunk
+// ahead, so that its memory latency overlaps the previous chunk's arithmetic.  Whole
 // chunks run the level-2 re-run and the reverse sweep on FP32 pairs;
 // other chunks run each trajectory on its own with the scalar functions.
 // Shared-memory stage of the hand-off: [kStages][kSub / 4 blocks][2 trajectories][thread].
@@ -652,26 +544,6 @@ __device__ __forceinline__ uint4 *segment_words(const AdjArgs &a, int block, int
     return a.words + ((size_t)block * (size_t)a.per + (size_t)i) * (size_t)a.n_blk * (2 * kL1Threads) + threadIdx.x;
 }
 
-// Both kernels run `sub` blocks per tile, block j of a tile taking
-// its trajectories [j blockDim, (j + 1) blockDim): one trajectory per thread.
-__global__ void __launch_bounds__(kL1Threads) adjoint_level1_kernel(AdjArgs a, int64_t seg0, int sub) {
-    const Batch &b = a.b;
-    const int64_t seg = seg0 + blockIdx.y;
-    float4 *const slots = segment_slots(a, (int)blockIdx.y);
-    const int tile = a.tile0 + (int)blockIdx.x / sub;
-    const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
-    const int set = b.tile_set[tile];
-    const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
-    const int64_t s0 = seg * K;
-    if (s0 >= N) return;  // uniform over the block
-    const int64_t s1 = min(s0 + K, N);
-    const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, a.nz.dt);  // the forward's own coefficients
-    if (li >= b.tile_count[tile]) return;
-    const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
-    const StepStream ss = step_stream((uint64_t)idx + a.nz.traj_base, a.K);
-    level1_segment(a, slots, k, ss, idx, s0, s1, a.ck.ck[(size_t)dchk(seg, a.ck.n_slots, b.dbg) * T + idx]);
-}
-
 // Level 1 with two trajectories per thread (trajectories li and li +
 // blockDim.x of the block's 2 blockDim.x), `sub` blocks per tile.
 template <bool WORDS>
@@ -698,37 +570,6 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_level1_pair_kernel(AdjArgs
     level1_segment2<WORDS>(a, slots, segment_words<WORDS>(a, a.tile0 * sub + (int)blockIdx.x, (int)blockIdx.y), k, ss,
                            idx, second, s0, s1, a.ck.ck[(size_t)slot * T + idx[0]],
                            a.ck.ck[(size_t)slot * T + idx[1]]);
-}
-
-__global__ void __launch_bounds__(kRevThreads, ABP_ADJ_MIN_BLOCKS) adjoint_reverse_kernel(AdjArgs a, SegView sv,
-                                                                                          int64_t seg0, int n,
-                                                                                          int sub, int64_t window) {
-    const Batch &b = a.b;
-    const int tile = a.tile0 + (int)blockIdx.x / sub;
-    const int li = ((int)blockIdx.x % sub) * (int)blockDim.x + (int)threadIdx.x;
-    const int set = b.tile_set[tile];
-    const int64_t N = b.set_steps[set], K = a.ck.every, T = b.total_traj;
-    if (seg0 * K >= N) return;  // uniform over the block
-    const abp_params p = b.params[set];
-    const Coef<float> k = load_coef<float>(b.coef_f, b.params, set, a.nz.dt);  // the forward's own coefficients
-    const float dtf = (float)a.nz.dt;
-    const float kx = (float)(-2.0 * kPi / p.L);  // d phi / dx with the sign of d cos / d phi
-    if (li >= b.tile_count[tile]) return;
-    const int64_t idx = dchk(b.tile_first[tile] + li, T, b.dbg);
-    const StepStream ss = step_stream((uint64_t)idx + a.nz.traj_base, a.K);
-    for (int i = n - 1; i >= 0; --i) {
-        const int64_t seg = seg0 + i, s0 = seg * K;
-        if (s0 >= N) continue;
-        float4 l0 = sv.lam[idx];
-        // windowed adjoint: the window ending at step (seg + 1) K starts from zero
-        if (window > 0 && ((seg + 1) * K) % window == 0) l0 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        float lx = l0.x, lv = l0.y, le = l0.z;
-        float acc[6] = {0, 0, 0, 0, 0, 0};
-        reverse_chunks(a, segment_slots(a, i), k, ss, kx, dtf, idx, s0, min(s0 + K, N), lx, lv, le, acc);
-        sv.lam[idx] = make_float4(lx, lv, le, 0.0f);
-#pragma unroll
-        for (int q = 0; q < 6; ++q) sv.G[(size_t)q * T + idx] += (double)acc[q];
-    }
 }
 
 // The reverse kernel with two trajectories per thread (trajectories li and
@@ -1062,12 +903,11 @@ AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool state
 }
 
 // Bytes abp_backward may take for the Philox blocks that level 1 hands to the reverse sweep
-// (no hand-off where one segment's buffers do not fit): none unless the kernels are the
-// paired ones; ABP_ADJ_HANDOFF_BYTES if set (0: never); else half the free device memory
+// (no hand-off where one segment's buffers do not fit): ABP_ADJ_HANDOFF_BYTES if set (0: never); else half the free device memory
 // not already held by the scratch.
 double handoff_budget(const abp_ctx *ctx) {
     // both kernels must map blocks and threads to trajectories alike
-    if (!ABP_ADJ_L1_PAIRS || !ABP_ADJ_REV_PAIRS || kL1Threads != kRevPairThreads) return -1.0;
+    if (kL1Threads != kRevPairThreads) return -1.0;
     const char *env = getenv("ABP_ADJ_HANDOFF_BYTES");
     if (env && *env) return strtod(env, nullptr);
     size_t free_b = 0, total_b = 0;
@@ -1101,7 +941,7 @@ bool use_states(const abp_ctx *ctx, double budget) {
 }
 
 // Segments per launch: as many as this many bytes of buffers hold (one where a segment's
-// own buffers are larger), shared evenly over the launches.  A launch and its events cost
+// own buffers are larger, or the noise is drawn again), shared evenly over the launches.  A launch and its events cost
 // the host some 5 us and the device the start and the drain of its blocks, and level 1 of
 // several segments runs side by side: with short segments of small batches that is most
 // of the time.  Backward, one segment per launch against 128 MB: 19,684 trajectories x
@@ -1113,6 +953,7 @@ bool use_states(const abp_ctx *ctx, double budget) {
 #define ABP_ADJ_LAUNCH_BYTES (128 << 20)
 #endif
 int64_t segments_per_launch(const abp_ctx *ctx, bool words, bool states, double budget, int64_t n_seg) {
+    if (!words && !states) return 1;
     const AdjLayout L = adj_layout(ctx, words, 1, states);
     int64_t per = (int64_t)((states ? state_bytes() : (double)ABP_ADJ_LAUNCH_BYTES) /
                             (double)std::max<size_t>(L.sub + L.words, 1));
@@ -1227,9 +1068,8 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         const int64_t n_run = (n_seg + per - 1) / per;  // launches of each kernel
         // blocks per tile: tiles hold up to kThreads * ppt trajectories
         const int cap = kThreads * std::max(ctx->ppt, 1);
-        const int sub1 = ABP_ADJ_L1_PAIRS ? pair_blocks_per_tile(ctx, kL1Threads) : (cap + kL1Threads - 1) / kL1Threads;
-        const int sub2 = ABP_ADJ_REV_PAIRS ? pair_blocks_per_tile(ctx, kRevPairThreads)
-                                           : (cap + kRevThreads - 1) / kRevThreads;
+        const int sub1 = pair_blocks_per_tile(ctx, kL1Threads);
+        const int sub2 = pair_blocks_per_tile(ctx, kRevPairThreads);
         const int sub_st = (cap + kL1Threads - 1) / kL1Threads, sub_sw = (cap + kSweepThreads - 1) / kSweepThreads;
         // The tiles in two halves, each with its own pair of streams: a trajectory's sweep
         // depends on no other's, so while one half's launch of a segment drains (its last
@@ -1285,10 +1125,8 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             else if (words) {
                 aj.words = wbuf[j & 1];
                 adjoint_level1_pair_kernel<true><<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
-            } else if (ABP_ADJ_L1_PAIRS)
+            } else
                 adjoint_level1_pair_kernel<false><<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
-            else
-                adjoint_level1_kernel<<<g1, kL1Threads, 0, g.l1>>>(aj, j * per, sub1);
             record(g.l1_done[j & 1], g.l1);
         };
         auto reverse = [&](const Group &g, int64_t j) {
@@ -1300,14 +1138,13 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             if (states) {
                 adjoint_sweep_kernel<<<(unsigned)((g.t1 - g.t0) * sub_sw), kSweepThreads, 0, g.rev>>>(
                     as, sv, j * per, (int)segments(j), sub_sw, window);
-            } else if (ABP_ADJ_REV_PAIRS) {
+            } else {
                 if (words) as.words = wbuf[j & 1];
-                const auto kernel =
-                    words ? (per > 1 ? adjoint_reverse_pair_kernel<true, true> : adjoint_reverse_pair_kernel<true, false>)
-                          : (per > 1 ? adjoint_reverse_pair_kernel<false, true> : adjoint_reverse_pair_kernel<false, false>);
+                const auto kernel = !words    ? adjoint_reverse_pair_kernel<false, false>
+                                    : per > 1 ? adjoint_reverse_pair_kernel<true, true>
+                                              : adjoint_reverse_pair_kernel<true, false>;
                 kernel<<<g2, kRevPairThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
-            } else
-                adjoint_reverse_kernel<<<g2, kRevThreads, 0, g.rev>>>(as, sv, j * per, (int)segments(j), sub2, window);
+            }
             record(g.rev_done[j & 1], g.rev);
             ctx->launches += 2;
         };

@@ -51,7 +51,7 @@ def test_segments_per_launch(abp, monkeypatch, K, slots, window):
         states[n] = grads(abp, K, window)
     n_seg = -(-203 // K)
     for n, (launches, g, t) in [*out.items(), *states.items()]:
-        runs = -(-n_seg // n) if n else 1
+        runs = 1 if n is None else -(-n_seg // max(n, 1))  # drawing again: one by one
         assert launches == 2 * runs + 2  # level 1 and reverse per run, the tile and the set sums
         np.testing.assert_array_equal(g, out[1][1])
         np.testing.assert_array_equal(t, out[1][2])
