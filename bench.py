@@ -37,10 +37,11 @@ LANES_PER_SM = 128
 # DRAM bytes (read + write) per launch of the integrator on the 2,097,152-trajectory sweep grid,
 # from one ncu capture of that kernel (dram__bytes_read.sum + dram__bytes_write.sum).  Lockstep:
 # the state load/store of one window, independent of its length (captured at 2,000 steps).  Work
-# queue: the bench's own launch (10^5 steps in ten rounds of 10^4-step items), captured whole --
-# the later rounds re-read the state from L2, the writes include its write-backs.
-TRAFFIC_PER_LAUNCH = {"integrate_kernel<float,2>": (52479744 + 1671424, 2097152),
-                      "persistent_kernel<float,2>": (52659712 + 19994112, 2097152)}
+# queue: the bench's own launch (10^5 steps in rounds of 10^4- or 10^3-step items), captured whole
+# -- the later rounds re-read the state from L2, the writes include its write-backs.
+TRAFFIC_PER_LAUNCH = {("integrate_kernel<float,2>", 0): (52487168 + 1549312, 2097152),
+                      ("persistent_kernel<float,2>", 10_000): (53048320 + 20087552, 2097152),
+                      ("persistent_kernel<float,2>", 1_000): (52667136 + 111377408, 2097152)}
 
 
 def parse():
@@ -828,9 +829,10 @@ def main():
     achieved = N_ALG * ps_launch / kern_avg / 1e12
     kname = ("persistent_kernel<float,%d>" if queue else "integrate_kernel<float,%d>") % tuning["particles_per_thread"]
     traffic = None
-    # the work-queue figure holds for the launch it was taken from (items of 10^4 steps)
-    if kname in TRAFFIC_PER_LAUNCH and not args.small and (not queue or spl == 10_000):
-        b_cap, t_cap = TRAFFIC_PER_LAUNCH[kname]
+    # a work-queue figure holds for the launch it was taken from (its items' steps)
+    tkey = (kname, spl if queue else 0)
+    if tkey in TRAFFIC_PER_LAUNCH and not args.small:
+        b_cap, t_cap = TRAFFIC_PER_LAUNCH[tkey]
         traffic = b_cap * w.total_traj / t_cap
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "T lane-op/s", "frac": achieved / peak,
             "traffic": traffic, "traffic_unit": "bytes per launch", "kernel": kname, "n_alg_per_particle_step": N_ALG,
