@@ -672,8 +672,12 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_states_kernel(AdjArgs a, i
 // The sweep over the rows of a launch's n segments, one trajectory per thread in blocks of
 // one warp.  The rows of consecutive segments follow one another, so the copies into the
 // thread's own ring (cp.async, kRowGroups - 1 groups of kRowGroup rows ahead, no barrier:
-// a thread reads only what it copied) run on across segments.
-constexpr int kRowGroup = 8, kRowGroups = 8, kSweepThreads = 32;
+// a thread reads only what it copied) run on across segments.  A group's first reads and
+// their sines wait for shared memory, so longer groups are faster as long as the ring leaves
+// room for six warps on an SM (32 KB each): backward of 256 trajectories x 4,000 steps, K =
+// 64, 262 us with eight groups of 8, 235 with four of 16, 237 with three; of 16,384 x 4,000,
+// K = 200, 480, 468 and 516 us.
+constexpr int kRowGroup = 16, kRowGroups = 4, kSweepThreads = 32;
 
 __global__ void __launch_bounds__(kSweepThreads) adjoint_sweep_kernel(AdjArgs a, SegView sv, int64_t seg0, int n,
                                                                       int sub, int64_t window) {
@@ -921,12 +925,12 @@ double handoff_budget(const abp_ctx *ctx) {
 // Whether level 1 hands every step's state to the sweep (adjoint_states_kernel): batches of
 // at most kStateTraj trajectories whose segments fit ABP_ADJ_STATE_BYTES (0: never) and
 // the hand-off's budget.  Backward of the pair kernels against this: 256 trajectories x
-// 4,000 steps, K = 64, 482 -> 267 us; 8,000 x 2,000, K = 64, 333 -> 206, K = 333, 309 ->
-// 210; 8,192 x 4,000, K = 1,000, 487 -> 319; 16,384 x 4,000, K = 200, 869 -> 478; 32,768 x
-// 2,000, K = 64, 588 -> 505, K = 500, 526 -> 485: beyond that the SMs hold more warps than
-// the ring leaves room for and the rows' 32 bytes a step come from HBM.  Fewer bytes mean
-// more launches (128 MB: 249, 240 and 488 us for the second to fourth of these, 256 MB:
-// 217, 212 and 369).
+// 4,000 steps, K = 64, 482 -> 235 us; 8,000 x 2,000, K = 64, 333 -> 199, K = 333, 309 ->
+// 202; 8,192 x 4,000, K = 1,000, 487 -> 302; 16,384 x 4,000, K = 200, 869 -> 468; 24,576 x
+// 4,000, K = 1,000, 625 -> 600; 32,768 x 2,000, K = 64, 588 -> 491: beyond that the SMs
+// hold more warps than the ring leaves room for and the rows' 32 bytes a step come from
+// HBM.  Fewer bytes mean more launches (with groups of 8 rows and 512 MB 206, 210 and 319
+// us for the second to fourth of these, 256 MB 217, 212 and 369, 128 MB 249, 240 and 488).
 #ifndef ABP_ADJ_STATE_TRAJ
 #define ABP_ADJ_STATE_TRAJ 32768
 #endif
