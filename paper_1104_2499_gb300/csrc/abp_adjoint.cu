@@ -913,7 +913,7 @@ double handoff_budget(const abp_ctx *ctx) {
     // both kernels must map blocks and threads to trajectories alike
     if (kL1Threads != kRevPairThreads) return -1.0;
     const char *env = getenv("ABP_ADJ_HANDOFF_BYTES");
-    if (env && *env) return strtod(env, nullptr);
+    if (env && *env) return std::min(strtod(env, nullptr), 1e15);  // segment counts stay in 64 bits
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
