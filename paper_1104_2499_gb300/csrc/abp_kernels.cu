@@ -554,10 +554,15 @@ struct WsCons {
 
 // The slots that every producer the consumer waits on has written: each lane reads
 // one producer's counter, so that the reads take one shared-memory latency together
-// instead of one each.
+// instead of one each.  The reduction hands the values round but orders no memory;
+// the warp barrier after it does, so that what lane p acquired from producer p is
+// ordered before every lane's reads of the ring.
 __device__ __forceinline__ int32_t ws_filled(const WsCons &c) {
     const int lane = threadIdx.x & 31;
-    return (int32_t)__reduce_min_sync(0xffffffffu, (uint32_t)ld_acquire_cta(&c.r.filled[lane < c.np ? lane : 0]));
+    const uint32_t mine = (uint32_t)ld_acquire_cta(&c.r.filled[lane < c.np ? lane : 0]);
+    const int32_t filled = (int32_t)__reduce_min_sync(0xffffffffu, mine);
+    __syncwarp();
+    return filled;
 }
 
 // advance() with the noise taken from the ring (one trajectory per thread; the
