@@ -991,6 +991,9 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     if (ctx->g < ctx->max_steps) return set_err(ctx, ABP_ESTATE, "abp_backward before the integration completed");
     if (!ctx->ckpt_complete)
         return set_err(ctx, ABP_ESTATE, "abp_backward after abp_load: the checkpoints do not cover the run from step 0");
+    const PtrKind kw = dJ_dmean_v ? ptr_kind(dJ_dmean_v, ctx->device) : PtrKind::Host;
+    if (kw == PtrKind::OtherDevice) return set_err(ctx, ABP_EINVAL, "abp_backward: weights on another GPU");
+    ctx->adj_valid = false;  // until this call has enqueued all of its work: the scratch changes from here on
     const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
     const double budget = handoff_budget(ctx);
     bool states = use_states(ctx, budget);
@@ -1037,8 +1040,6 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     cudaError_t e = cudaSuccess;
     const double *w = nullptr;
     if (dJ_dmean_v) {
-        const PtrKind kw = ptr_kind(dJ_dmean_v, ctx->device);
-        if (kw == PtrKind::OtherDevice) return set_err(ctx, ABP_EINVAL, "abp_backward: weights on another GPU");
         if (kw == PtrKind::Device) {
             w = dJ_dmean_v;
         } else {

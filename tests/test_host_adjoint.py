@@ -1,0 +1,118 @@
+"""Host side of the adjoint on the CPU: the library's objects linked with a CUDA runtime that runs
+no kernel, notes every launch and its stream, and lets named calls fail (tests/helpers/
+fake_cudart.cpp).  Each test is a child process with that library in place of libabp.so."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SRC = os.path.join(ROOT, "tests", "helpers", "fake_cudart.cpp")
+
+PRELUDE = r'''
+import ctypes, os, sys
+import numpy as np
+sys.path.insert(0, os.environ["ABP_ROOT"])
+from paper_1104_2499_gb300 import abp as A, workloads as W
+
+L = A.lib()
+L.fake_fail.argtypes = [ctypes.c_char_p, ctypes.c_long, ctypes.c_long]
+L.fake_kernel.argtypes, L.fake_kernel.restype = [ctypes.c_long], ctypes.c_char_p
+L.fake_ordered.argtypes = [ctypes.c_void_p, ctypes.c_long]
+for f in ("fake_calls", "fake_launches", "fake_live", "fake_peak"):
+    getattr(L, f).restype = ctypes.c_size_t if f in ("fake_live", "fake_peak") else ctypes.c_long
+
+
+def integrated(n_traj=(300, 65, 1), n_steps=(203, 64, 7), K=8, ppt=2):
+    n = len(n_traj)
+    w = W.Workload(name="host", sets=[W.params(D=0.1)] * n, n_traj=list(n_traj), n_steps=list(n_steps), dt=1e-3, seed=1,
+                   checkpoint_every=K)
+    ctx = A.abp_create(A.make_config(w, particles_per_thread=ppt, schedule=1, steps_per_launch=max(n_steps)))
+    A.abp_set_params(ctx, w.sets, w.n_traj, w.n_steps)
+    A.abp_integrate(ctx)
+    return ctx, np.zeros((n, 6)), np.zeros((sum(n_traj), 6))
+
+
+def status(call, *a):
+    try:
+        call(*a)
+    except A.AbpError as e:
+        return e.status
+    return A.ABP_OK
+
+
+def kernels(i):
+    return [L.fake_kernel(k).decode() for k in range(i, L.fake_launches())]
+'''
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    from paper_1104_2499_gb300 import build as B
+
+    try:
+        nvcc = B.nvcc()
+    except RuntimeError:
+        pytest.skip("nvcc not available to build libabp.so")
+    if not shutil.which("g++"):
+        pytest.skip("no C++ compiler")
+    B.build()
+    tmp = tmp_path_factory.mktemp("fake")
+    lib = str(tmp / "libabp_fake.so")
+    objs = [os.path.join(B.OUT, s.replace(".cu", ".o")) for s in B.SOURCES]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-fPIC", "-shared", "-o", lib, SRC] + objs +
+                   ["-I", os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include"), "-Wl,-Bsymbolic",
+                    "-Wl,-z,defs", "-ldl", "-lpthread", "-lrt"], check=True)
+
+    def run(code, **env):
+        e = {k: v for k, v in os.environ.items() if not k.startswith("ABP_")}
+        e.update(ABP_LIB=lib, ABP_ROOT=ROOT, **env)
+        r = subprocess.run([sys.executable, "-c", PRELUDE + code], env=e, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stderr[-4000:]
+
+    return run
+
+
+def test_readout_follows_a_backward(child):
+    child('''
+ctx, grad, dv = integrated()
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_ESTATE
+A.abp_backward(ctx, None, grad)
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_OK
+# a call refused for its arguments leaves the sums of the last one readable
+assert status(A.abp_backward, ctx, None, None) == A.ABP_EINVAL
+assert status(A.abp_backward, ctx, None, grad, 7) == A.ABP_EINVAL
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_OK
+''')
+
+
+# small buffers first (the noise drawn again), then a larger form that finds no memory at all
+def test_readout_is_refused_after_a_backward_without_scratch(child):
+    child('''
+os.environ["ABP_ADJ_HANDOFF_BYTES"] = "0"
+ctx, grad, dv = integrated()
+A.abp_backward(ctx, None, grad)
+del os.environ["ABP_ADJ_HANDOFF_BYTES"]
+L.fake_fail(b"cudaMalloc", 0, 1000)
+assert status(A.abp_backward, ctx, None, grad) == A.ABP_ENOMEM
+L.fake_fail(None, 0, 0)
+n = L.fake_launches()
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_ESTATE
+assert L.fake_launches() == n  # no kernel on a scratch that is gone
+A.abp_backward(ctx, None, grad)
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_OK
+''')
+
+
+@pytest.mark.parametrize("call", ["cudaMemsetAsync", "cudaEventRecord", "cudaStreamWaitEvent", "launch", "cudaMemcpyAsync"])
+def test_readout_is_refused_after_a_backward_that_broke_off(child, call):
+    child('''
+ctx, grad, dv = integrated()
+A.abp_backward(ctx, None, grad)
+L.fake_fail(CALL, 0, 1000)
+assert status(A.abp_backward, ctx, None, grad) == A.ABP_ECUDA
+L.fake_fail(None, 0, 0)
+assert status(A.abp_backward_traj, ctx, dv) == A.ABP_ESTATE
+'''.replace("CALL", repr(call.encode())))
