@@ -854,6 +854,7 @@ abp_status set_err(abp_ctx *ctx, abp_status st, const char *msg, cudaError_t e =
     if (e != cudaSuccess) {
         ctx->err += ": ";
         ctx->err += cudaGetErrorString(e);
+        cudaGetLastError();  // reported here: the next call's launch check must not find it again
     }
     return st;
 }

@@ -37,6 +37,7 @@ abp_status fail(abp_ctx *ctx, abp_status st, const char *fmt, ...) {
 }
 
 abp_status cuda_fail(abp_ctx *ctx, cudaError_t e, const char *what) {
+    cudaGetLastError();  // reported here: the next call's launch check must not find it again
     return fail(ctx, e == cudaErrorMemoryAllocation ? ABP_ENOMEM : ABP_ECUDA, "%s: %s (%s)", what,
                 cudaGetErrorName(e), cudaGetErrorString(e));
 }

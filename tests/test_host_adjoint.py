@@ -116,3 +116,25 @@ assert status(A.abp_backward, ctx, None, grad) == A.ABP_ECUDA
 L.fake_fail(None, 0, 0)
 assert status(A.abp_backward_traj, ctx, dv) == A.ABP_ESTATE
 '''.replace("CALL", repr(call.encode())))
+
+
+# the runtime keeps a failed call's error until it is asked for: a call that reported it has to
+# take it away, or the next one, which checks its launches by it, reports it a second time
+@pytest.mark.parametrize("call", ["cudaMemsetAsync", "cudaEventRecord", "cudaStreamWaitEvent"])
+def test_an_error_is_reported_by_one_call_only(child, call):
+    child('''
+ctx, grad, dv = integrated()
+L.fake_fail(CALL, 0, 1)
+first = status(A.abp_backward, ctx, None, grad)
+if CALL == b"cudaMemsetAsync":  # the work queue clears its counters too
+    assert first == A.ABP_ECUDA
+    w = W.Workload(name="q", sets=[W.params()], n_traj=[600], n_steps=[100], dt=1e-3, seed=1)
+    q = A.abp_create(A.make_config(w, particles_per_thread=2, schedule=2, steps_per_launch=50))
+    A.abp_set_params(q, w.sets, w.n_traj, w.n_steps)
+    L.fake_fail(CALL, 0, 1)
+    assert status(A.abp_integrate, q) == A.ABP_ECUDA
+    A.abp_reset(q, 1)
+    assert status(A.abp_integrate, q) == A.ABP_OK
+assert first == A.ABP_ECUDA
+assert status(A.abp_backward, ctx, None, grad) == A.ABP_OK
+'''.replace("CALL", repr(call.encode())))
