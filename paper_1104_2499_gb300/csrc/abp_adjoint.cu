@@ -1121,6 +1121,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         // reader of that buffer, has finished
         auto segments = [&](int64_t j) { return (unsigned)std::min(per, n_seg - j * per); };
         auto level1 = [&](const Group &g, int64_t j) {
+            if (e != cudaSuccess) return;  // nothing is launched whose order is not established
             AdjArgs aj = a;
             aj.sub = sub[j & 1];
             aj.tile0 = g.t0;
@@ -1137,6 +1138,7 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         };
         auto reverse = [&](const Group &g, int64_t j) {
             wait(g.rev, g.l1_done[j & 1]);
+            if (e != cudaSuccess) return;
             AdjArgs as = a;
             as.sub = sub[j & 1];
             as.tile0 = g.t0;
@@ -1168,10 +1170,18 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
                 }
                 reverse(grp[g], j);
             }
-        for (int g = 1; g < n_grp; ++g) {  // also after an error: the caller's stream then follows all launches
-            cudaEventRecord(end, grp[g].rev);
-            cudaStreamWaitEvent(s, end, 0);
-        }
+        // The caller's stream follows all launches: it waits for the sweeps' streams, which have
+        // waited for their level-1 streams, and after an error for those as well (on the host
+        // where an event cannot be used).
+        auto join = [&](cudaStream_t st) {
+            cudaError_t je = cudaEventRecord(end, st);
+            if (je == cudaSuccess) je = cudaStreamWaitEvent(s, end, 0);
+            if (je != cudaSuccess) cudaStreamSynchronize(st);
+            if (e == cudaSuccess) e = je;
+        };
+        for (int g = 1; g < n_grp; ++g) join(grp[g].rev);
+        if (e != cudaSuccess)
+            for (int g = 0; g < n_grp; ++g) join(grp[g].l1);
         if (e != cudaSuccess) return set_err(ctx, ABP_ECUDA, "abp_backward: launch", e);
         adjoint_final_kernel<<<ctx->n_tiles, kThreads, 0, s>>>(a, sv);
         ctx->launches += 1;

@@ -138,3 +138,36 @@ if CALL == b"cudaMemsetAsync":  # the work queue clears its counters too
 assert first == A.ABP_ECUDA
 assert status(A.abp_backward, ctx, None, grad) == A.ABP_OK
 '''.replace("CALL", repr(call.encode())))
+
+
+# one group of tiles and two; state rows in one launch and in several, the noise hand-off, the
+# noise drawn again
+@pytest.mark.parametrize("sms", [152, 2])
+@pytest.mark.parametrize("form", [{}, {"ABP_ADJ_STATE_BYTES": "700000"},
+                                  {"ABP_ADJ_STATE_BYTES": "0", "ABP_ADJ_HANDOFF_BYTES": "200000"},
+                                  {"ABP_ADJ_HANDOFF_BYTES": "0"}], ids=["states", "states-several", "handoff", "redraw"])
+def test_the_callers_stream_follows_every_launch(child, sms, form):
+    # whichever call fails, and whether once or from then on, the caller's stream is ordered after
+    # every kernel that was launched, and a failure is never reported as success
+    child('''
+L.fake_sms(SMS)
+ctx, grad, dv = integrated(K=24)
+A.abp_backward(ctx, None, grad)  # streams, events and scratch are there
+names = set()
+for call in (b"none", b"cudaEventRecord", b"cudaStreamWaitEvent", b"launch"):
+    for n in (1, 1000):
+        i, more = 0, True
+        while more:
+            n0 = L.fake_launches()
+            L.fake_fail(call, i, n)
+            s = status(A.abp_backward, ctx, None, grad)
+            more = L.fake_calls() > i
+            L.fake_fail(None, 0, 0)
+            assert s == (A.ABP_ECUDA if more else A.ABP_OK), (call, i, n, s)
+            for k in range(n0, L.fake_launches()):
+                assert L.fake_ordered(None, k), (call, i, n, k - n0, L.fake_kernel(k))
+            names |= set(kernels(n0))
+            i += 1
+        assert i > (0 if call == b"none" else 2)
+assert any(KERNEL in k for k in names), names
+'''.replace("SMS", str(sms)).replace("KERNEL", repr("level1_pair" if "ABP_ADJ_HANDOFF_BYTES" in form else "states")), **form)
