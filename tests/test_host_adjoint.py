@@ -171,3 +171,28 @@ for call in (b"none", b"cudaEventRecord", b"cudaStreamWaitEvent", b"launch"):
         assert i > (0 if call == b"none" else 2)
 assert any(KERNEL in k for k in names), names
 '''.replace("SMS", str(sms)).replace("KERNEL", repr("level1_pair" if "ABP_ADJ_HANDOFF_BYTES" in form else "states")), **form)
+
+
+# the form a batch takes: every step's state up to 32,768 trajectories and 512 MB of buffers, else
+# the noise hand-off within its budget, else the noise drawn again; a launch over several segments
+# has its own sweep
+@pytest.mark.parametrize("n_traj,K,env,expect", [
+    (32768, 24, {}, ["adjoint_states_kernel", "adjoint_sweep_kernel"]),
+    (32769, 24, {}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
+    (32768, 24, {"ABP_ADJ_STATE_BYTES": "0"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
+    (366, 24, {"ABP_ADJ_STATE_BYTES": "1"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
+    (366, 300, {"ABP_ADJ_STATE_BYTES": "0"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb0"]),
+    (366, 24, {"ABP_ADJ_STATE_BYTES": "0", "ABP_ADJ_HANDOFF_BYTES": "0"},
+     ["adjoint_level1_pair_kernelILb0", "adjoint_reverse_pair_kernelILb0ELb0"]),
+    (366, 24, {"ABP_ADJ_HANDOFF_BYTES": "0"}, ["adjoint_level1_pair_kernelILb0", "adjoint_reverse_pair_kernelILb0ELb0"]),
+])
+def test_the_kernels_each_form_launches(child, n_traj, K, env, expect):
+    child('''
+ctx, grad, dv = integrated(n_traj=(N,), n_steps=(203,), K=KK)
+n0 = L.fake_launches()
+A.abp_backward(ctx, None, grad)
+ks = kernels(n0)
+assert "adjoint_final_kernel" in ks[-2] and "adjoint_set_kernel" in ks[-1], ks
+names = EXPECT
+assert all(any(n in k for n in names) for k in ks[:-2]) and all(any(n in k for k in ks) for n in names), ks
+'''.replace("KK", str(K)).replace("(N,)", "(%d,)" % n_traj).replace("EXPECT", repr(expect)), **env)
