@@ -248,8 +248,9 @@ ABP_API abp_status abp_load(abp_ctx *ctx, const void *buf, size_t bytes);
  * checkpoint_every; 8 bytes per trajectory per step of checkpoint_every for
  * handing the noise of each interval's first re-run to its reverse sweep, if that
  * fits in the budget the environment variable ABP_ADJ_HANDOFF_BYTES gives (0:
- * never), by default half the free device memory -- else the noise is drawn
- * again; short intervals are taken several at a time, up to 128 MB in all.
+ * never), by default half the free device memory (asked for when the scratch has
+ * to grow) -- else the noise is drawn again; short intervals are taken several at
+ * a time, up to 128 MB in all.
  * Batches of at most 32,768 trajectories take 32 bytes per trajectory per step
  * instead, for as many intervals as 512 MB hold (ABP_ADJ_STATE_BYTES; 0: never),
  * within the same budget.  Where an allocation fails the smaller forms are used

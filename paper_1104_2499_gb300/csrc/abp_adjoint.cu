@@ -914,14 +914,20 @@ AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool state
     return L;
 }
 
-// Bytes abp_backward may take for the Philox blocks that level 1 hands to the reverse sweep
-// (no hand-off where one segment's buffers do not fit): ABP_ADJ_HANDOFF_BYTES if set (0: never); else half the free device memory
-// not already held by the scratch.
-double handoff_budget(const abp_ctx *ctx) {
-    // both kernels must map blocks and threads to trajectories alike
-    if (kL1Threads != kRevPairThreads) return -1.0;
+// both kernels must map blocks and threads to trajectories alike for the hand-off
+static_assert(kL1Threads == kRevPairThreads, "level 1 and the reverse sweep share a block's trajectories");
+
+// Bytes abp_backward may take for what level 1 hands to the reverse sweep (no hand-off where one
+// segment's buffers do not fit): ABP_ADJ_HANDOFF_BYTES (0: never) ...
+bool handoff_env(double *budget) {
     const char *env = getenv("ABP_ADJ_HANDOFF_BYTES");
-    if (env && *env) return std::min(strtod(env, nullptr), 1e15);  // segment counts stay in 64 bits
+    if (!env || !*env) return false;
+    *budget = std::min(strtod(env, nullptr), 1e15);  // segment counts stay in 64 bits
+    return true;
+}
+
+// ... else half the free device memory, the scratch's own counted as free.
+double handoff_memory(const abp_ctx *ctx) {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         cudaGetLastError();
@@ -976,6 +982,34 @@ int64_t segments_per_launch(const abp_ctx *ctx, bool words, bool states, double 
     return launches > 0 ? (n_seg + launches - 1) / launches : 1;
 }
 
+// The form of a backward call and its scratch: every step's state, the noise hand-off or
+// (neither) the noise drawn again, and the segments of a launch.
+struct AdjForm {
+    bool states, words;
+    int64_t per;
+    AdjLayout L;
+};
+
+AdjForm form_within(const abp_ctx *ctx, int64_t n_seg, double budget) {
+    AdjForm f;
+    f.states = use_states(ctx, budget);
+    f.words = !f.states && (double)adj_layout(ctx, true).words <= budget;
+    f.per = segments_per_launch(ctx, f.words, f.states, budget, n_seg);
+    f.L = adj_layout(ctx, f.words, f.per, f.states);
+    return f;
+}
+
+// Without a budget from the environment the free memory is asked for only where the
+// scratch has to grow: the query takes the host some 18 us, a tenth of a short backward
+// (33,000 trajectories x 500 steps, K = 500: 155 us with it on every call, 137 without;
+// 300 x 1,000, K = 64: 114 and 94).
+AdjForm choose_form(const abp_ctx *ctx, int64_t n_seg) {
+    double budget = 1e15;
+    const bool env = handoff_env(&budget);
+    const AdjForm f = form_within(ctx, n_seg, budget);
+    return env || (ctx->d_adj.p && f.L.need <= ctx->d_adj.cap) ? f : form_within(ctx, n_seg, handoff_memory(ctx));
+}
+
 }  // namespace
 }  // namespace abp
 
@@ -1003,12 +1037,11 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
     if (kw == PtrKind::OtherDevice) return set_err(ctx, ABP_EINVAL, "abp_backward: weights on another GPU");
     ctx->adj_valid = false;  // until this call has enqueued all of its work: the scratch changes from here on
     const int64_t n_sub = sub_slots(ctx->cfg.checkpoint_every);
-    const double budget = handoff_budget(ctx);
-    bool states = use_states(ctx, budget);
-    bool words = !states && (double)adj_layout(ctx, true).words <= budget;
     const int64_t Kc = ctx->cfg.checkpoint_every, n_seg = (ctx->max_steps + Kc - 1) / Kc;
-    int64_t per = segments_per_launch(ctx, words, states, budget, n_seg);
-    AdjLayout L = adj_layout(ctx, words, per, states);
+    AdjForm form = choose_form(ctx, n_seg);
+    bool &states = form.states, &words = form.words;
+    int64_t &per = form.per;
+    AdjLayout &L = form.L;
     DevBuf &sc = ctx->d_adj;
     if (!sc.p || sc.cap < L.need) {
         sc.release();

@@ -186,6 +186,7 @@ cudaError_t cudaFreeHost(void *p) {
     return cudaSuccess;
 }
 cudaError_t cudaMemGetInfo(size_t *f, size_t *t) {
+    if (fails("cudaMemGetInfo")) return err(cudaErrorUnknown);
     *f = g_total - g_live;
     *t = g_total;
     return cudaSuccess;

@@ -196,3 +196,26 @@ assert "adjoint_final_kernel" in ks[-2] and "adjoint_set_kernel" in ks[-1], ks
 names = EXPECT
 assert all(any(n in k for n in names) for k in ks[:-2]) and all(any(n in k for k in ks) for n in names), ks
 '''.replace("KK", str(K)).replace("(N,)", "(%d,)" % n_traj).replace("EXPECT", repr(expect)), **env)
+
+
+# the query takes longer than a short backward's launches: only a scratch that has to grow asks
+@pytest.mark.parametrize("K", [8, 50])
+@pytest.mark.parametrize("form", [{}, {"ABP_ADJ_STATE_BYTES": "0"}], ids=["states", "handoff"])
+def test_free_memory_is_asked_for_only_to_grow_the_scratch(child, form, K):
+    child('''
+ctx, grad, dv = integrated(K=KK)
+L.fake_fail(b"cudaMemGetInfo", 0, 0)
+A.abp_backward(ctx, None, grad)
+assert L.fake_calls() == 1
+n0 = L.fake_launches()
+A.abp_backward(ctx, None, grad)
+assert L.fake_calls() == 1
+again = kernels(n0)
+# a query that fails leaves the smallest form
+ctx, grad, dv = integrated(K=KK)
+L.fake_fail(b"cudaMemGetInfo", 0, 1)
+n0 = L.fake_launches()
+A.abp_backward(ctx, None, grad)
+assert L.fake_calls() == 1 and any("reverse_pair_kernelILb0ELb0" in k for k in kernels(n0)), kernels(n0)
+assert not any("ILb0ELb0" in k for k in again), again
+'''.replace("KK", str(K)), **form)
