@@ -949,12 +949,16 @@ double handoff_memory(const abp_ctx *ctx) {
 #define ABP_ADJ_STATE_TRAJ 32768
 #endif
 constexpr int64_t kStateTraj = ABP_ADJ_STATE_TRAJ;
+// A run of one segment has no other to step beside it in level 1, so there the rows' traffic
+// counts earlier: one backward of 500 steps, K = 500, 16,384 trajectories 106 us against 127
+// with the hand-off, 20,000 119 against 127, 24,576 129 against 128, 32,768 153 against 135.
+constexpr int64_t kStateTrajOne = 24576;
 double state_bytes() {
     const char *env = getenv("ABP_ADJ_STATE_BYTES");
     return env && *env ? std::min(strtod(env, nullptr), 4e9) : 512.0 * (1 << 20);  // row numbers stay in 32 bits
 }
-bool use_states(const abp_ctx *ctx, double budget) {
-    return ctx->total_traj <= kStateTraj &&
+bool use_states(const abp_ctx *ctx, int64_t n_seg, double budget) {
+    return ctx->total_traj <= (n_seg > 1 ? kStateTraj : kStateTrajOne) &&
            (double)adj_layout(ctx, false, 1, true).sub <= std::min(budget, state_bytes());
 }
 
@@ -992,7 +996,7 @@ struct AdjForm {
 
 AdjForm form_within(const abp_ctx *ctx, int64_t n_seg, double budget) {
     AdjForm f;
-    f.states = use_states(ctx, budget);
+    f.states = use_states(ctx, n_seg, budget);
     f.words = !f.states && (double)adj_layout(ctx, true).words <= budget;
     f.per = segments_per_launch(ctx, f.words, f.states, budget, n_seg);
     f.L = adj_layout(ctx, f.words, f.per, f.states);

@@ -173,13 +173,17 @@ assert any(KERNEL in k for k in names), names
 '''.replace("SMS", str(sms)).replace("KERNEL", repr("level1_pair" if "ABP_ADJ_HANDOFF_BYTES" in form else "states")), **form)
 
 
-# the form a batch takes: every step's state up to 32,768 trajectories and 512 MB of buffers, else
+# the form a batch takes: every step's state up to 32,768 trajectories (24,576 where the run is one
+# segment) and 512 MB of buffers, else
 # the noise hand-off within its budget, else the noise drawn again; a launch over several segments
 # has its own sweep
 @pytest.mark.parametrize("n_traj,K,env,expect", [
     (32768, 24, {}, ["adjoint_states_kernel", "adjoint_sweep_kernel"]),
     (32769, 24, {}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
     (32768, 24, {"ABP_ADJ_STATE_BYTES": "0"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
+    (24576, 300, {}, ["adjoint_states_kernel", "adjoint_sweep_kernel"]),
+    (24577, 300, {}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb0"]),
+    (24577, 200, {}, ["adjoint_states_kernel", "adjoint_sweep_kernel"]),
     (366, 24, {"ABP_ADJ_STATE_BYTES": "1"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb1"]),
     (366, 300, {"ABP_ADJ_STATE_BYTES": "0"}, ["adjoint_level1_pair_kernelILb1", "adjoint_reverse_pair_kernelILb1ELb0"]),
     (366, 24, {"ABP_ADJ_STATE_BYTES": "0", "ABP_ADJ_HANDOFF_BYTES": "0"},
