@@ -253,9 +253,10 @@ ABP_API abp_status abp_load(abp_ctx *ctx, const void *buf, size_t bytes);
  * a time, up to 128 MB in all.
  * Batches of at most 32,768 trajectories (24,576 where checkpoint_every covers the
  * whole run) take 32 bytes per trajectory per step instead, for as many intervals as
- * 512 MB hold (ABP_ADJ_STATE_BYTES; 0: never), within the same budget.  Where an allocation fails the smaller forms are used
- * (one interval at a time, then the noise drawn again).  The results are the
- * same bit for bit either way. */
+ * 512 MB hold (ABP_ADJ_STATE_BYTES; 0: never), within the same budget.  Where all
+ * intervals fit at once one buffer of two is taken: half of these.  Where an
+ * allocation fails the smaller forms are used (one interval at a time, then the
+ * noise drawn again).  The results are the same bit for bit either way. */
 ABP_API abp_status abp_backward(abp_ctx *ctx, const double *dJ_dmean_v, double *grad);
 
 /* Windowed pathwise adjoint: as abp_backward, with the adjoint state restarted

@@ -867,9 +867,10 @@ abp_status set_err(abp_ctx *ctx, abp_status st, const char *msg, cudaError_t e =
 }
 
 // Scratch of abp_backward, one allocation: the tile partials, the set gradients, the
-// weights, lambda, the per-trajectory sums, then the two sub-checkpoint buffers and,
-// last, the two Philox-block buffers of the hand-off (0 bytes without it), each for
-// `per` segments.  abp_backward_traj reads lambda and the sums of the last call at the
+// weights, lambda, the per-trajectory sums, then the sub-checkpoint buffers and,
+// last, the Philox-block buffers of the hand-off (0 bytes without it), each for
+// `per` segments: two, alternating by launch, or one where a launch covers every
+// segment.  abp_backward_traj reads lambda and the sums of the last call at the
 // same offsets, which depend on neither.
 struct AdjLayout {
     size_t sub1, sub, part, grad, w, lam, g, words1, words, need;
@@ -889,12 +890,12 @@ int pair_blocks_per_tile(const abp_ctx *ctx, int threads) {
     return (cap + 2 * threads - 1) / (2 * threads);
 }
 
-AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool states = false) {
+AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool states = false, int buffers = 2) {
     AdjLayout L;
     const int64_t T = ctx->total_traj, Kc = ctx->cfg.checkpoint_every;
     const int64_t n_sub = states ? Kc : sub_slots(Kc);
     L.sub1 = sizeof(float4) * (size_t)(per * n_sub) * (size_t)T;
-    L.sub = 2 * align256(L.sub1);  // two buffers, alternating by launch
+    L.sub = buffers * align256(L.sub1);
     L.part = sizeof(double) * 6 * (size_t)std::max(ctx->n_tiles, 1);
     L.grad = sizeof(double) * 6 * (size_t)std::max(ctx->n_sets, 1);
     L.w = sizeof(double) * (size_t)std::max(ctx->n_sets, 1);
@@ -902,7 +903,7 @@ AdjLayout adj_layout(const abp_ctx *ctx, bool words, int64_t per = 1, bool state
     L.g = sizeof(double) * 6 * (size_t)std::max<int64_t>(T, 1);
     const size_t blocks = (size_t)ctx->n_tiles * (size_t)pair_blocks_per_tile(ctx, kL1Threads);
     L.words1 = words ? sizeof(uint4) * blocks * (size_t)(per * n_sub * (kSub / 4)) * 2 * kL1Threads : 0;
-    L.words = 2 * align256(L.words1);
+    L.words = buffers * align256(L.words1);
     L.off_part = 0;
     L.off_grad = L.off_part + align256(L.part);
     L.off_w = L.off_grad + align256(L.grad);
@@ -999,7 +1000,7 @@ AdjForm form_within(const abp_ctx *ctx, int64_t n_seg, double budget) {
     f.states = use_states(ctx, n_seg, budget);
     f.words = !f.states && (double)adj_layout(ctx, true).words <= budget;
     f.per = segments_per_launch(ctx, f.words, f.states, budget, n_seg);
-    f.L = adj_layout(ctx, f.words, f.per, f.states);
+    f.L = adj_layout(ctx, f.words, f.per, f.states, f.per < n_seg ? 2 : 1);
     return f;
 }
 
@@ -1054,13 +1055,13 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
             cudaGetLastError();
             per = 1;
             states = false;
-            L = adj_layout(ctx, words);
+            L = adj_layout(ctx, words, per, states, n_seg > 1 ? 2 : 1);
             e = cudaMalloc(&sc.p, L.need);
         }
         if (e != cudaSuccess && words) {  // no room for the hand-off: draw the blocks twice instead
             cudaGetLastError();
             words = false;
-            L = adj_layout(ctx, false);
+            L = adj_layout(ctx, words, per, states, n_seg > 1 ? 2 : 1);
             e = cudaMalloc(&sc.p, L.need);
         }
         if (e != cudaSuccess) {
@@ -1130,16 +1131,12 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         // of two).  A batch with fewer blocks than SMs runs in one group: it leaves SMs
         // free anyway, and each launch costs host time.
         const int n_grp = !states && ctx->n_tiles >= 2 && (int64_t)ctx->n_tiles * sub2 >= ctx->sm_count ? kAdjGroups : 1;
-        if (!ctx->adj_stream[0]) {
-            for (int i = 0; e == cudaSuccess && i < 2 * kAdjGroups - 1; ++i)
-                e = cudaStreamCreateWithFlags(&ctx->adj_stream[i], cudaStreamNonBlocking);
-            for (int i = 0; e == cudaSuccess && i < abp_ctx::kAdjEvents; ++i)
-                e = cudaEventCreateWithFlags(&ctx->adj_ev[i], cudaEventDisableTiming);
-            if (e != cudaSuccess) {
-                ctx->release_streams();
-                return set_err(ctx, ABP_ECUDA, "abp_backward: stream set-up", e);
-            }
-        }
+        // the groups' streams and events, kept for the next call
+        for (int i = 0; e == cudaSuccess && i < 2 * n_grp - 1; ++i)
+            if (!ctx->adj_stream[i]) e = cudaStreamCreateWithFlags(&ctx->adj_stream[i], cudaStreamNonBlocking);
+        for (int i = 0; e == cudaSuccess && i < 2 + 4 * n_grp; ++i)
+            if (!ctx->adj_ev[i]) e = cudaEventCreateWithFlags(&ctx->adj_ev[i], cudaEventDisableTiming);
+        if (e != cudaSuccess) return set_err(ctx, ABP_ECUDA, "abp_backward: stream set-up", e);
         struct Group {
             cudaStream_t rev, l1;
             cudaEvent_t *l1_done, *rev_done;  // [2] by launch parity

@@ -223,3 +223,36 @@ A.abp_backward(ctx, None, grad)
 assert L.fake_calls() == 1 and any("reverse_pair_kernelILb0ELb0" in k for k in kernels(n0)), kernels(n0)
 assert not any("ILb0ELb0" in k for k in again), again
 '''.replace("KK", str(K)), **form)
+
+
+# what a call takes and keeps: one buffer where one launch covers every segment, the streams and
+# events of the groups in use
+@pytest.mark.parametrize("form,step_bytes", [({}, 16), ({"ABP_ADJ_STATE_BYTES": "0"}, 0)], ids=["states", "handoff"])
+def test_one_launch_takes_one_buffer(child, form, step_bytes):
+    child('''
+ctx, grad, dv = integrated(n_traj=(3000,), n_steps=(200,), K=40)
+before, streams, events = L.fake_live(), L.fake_streams(), L.fake_events()
+n0 = L.fake_launches()
+A.abp_backward(ctx, None, grad)
+assert len(kernels(n0)) == 4, kernels(n0)
+used = L.fake_live() - before
+if STEP:
+    rows = STEP * 200 * 3000
+else:  # five segments of 5 sub-checkpoints and 10 blocks of noise for the 12 blocks of 2 x 128 trajectories
+    rows = 5 * 5 * 16 * 3000 + 12 * 5 * 10 * 2 * 128 * 16
+# and 64 bytes per trajectory, the tile and set sums, each rounded to 256 bytes
+assert rows + 64 * 3000 <= used <= rows + 64 * 3000 + 48 * 6 + 56 + 8 * 256, (used, rows)
+assert (L.fake_streams() - streams, L.fake_events() - events) == (1, 6)
+A.abp_backward(ctx, None, grad)
+assert (L.fake_streams() - streams, L.fake_events() - events) == (1, 6)
+# a batch of two groups adds the second one's, and a set-up that fails keeps what there was
+L.fake_sms(2)
+ctx, grad, dv = integrated(n_traj=(40000,), n_steps=(200,), K=40)
+L.fake_fail(b"cudaEventCreateWithFlags", 3, 1)
+assert status(A.abp_backward, ctx, None, grad) == A.ABP_ECUDA
+L.fake_fail(None, 0, 0)
+A.abp_backward(ctx, None, grad)
+assert (L.fake_streams() - streams, L.fake_events() - events) == (1 + 3, 6 + 10)
+A.abp_destroy(ctx)
+assert (L.fake_streams() - streams, L.fake_events() - events) == (1, 6)
+'''.replace("STEP", str(step_bytes)), **form)
