@@ -415,13 +415,16 @@ constexpr int group_unroll() {
 // one-trajectory sets x 3,164 steps 191 -> 146 us, 20,000 trajectories of one set x 1,659
 // steps 88 -> 82 us, 53 sets of 829 on the work queue 557 -> 488 us).  Two or three blocks
 // are no faster there, and slower where tiles are nearly empty and blocks per SM count
-// (2,000 sets of 20 on the work queue: 471 us, 859 and 599 with two and three).
+// (2,000 sets of 20 on the work queue: 471 us, 859 and 599 with two and three).  Not so the
+// lockstep kernel of Heun's scheme, whose longer body wants more than 64 registers: told
+// nothing, 100,000 trajectories x 1,000 steps take 222 us against 236, 400,000 743 against
+// 805, 30,000 95 against 99 (packed tiles and the work queue: the same either way).
 #ifndef ABP_BLOCKS_XS2
 #define ABP_BLOCKS_XS2 4
 #endif
-template <typename R, int PPT, int MODE, bool PACKED = false>
+template <typename R, int PPT, int MODE, bool PACKED, bool QUEUE>
 constexpr int min_blocks() {
-    if (sizeof(R) == 4 && PPT == 1) return 4;
+    if (sizeof(R) == 4 && PPT == 1) return MODE == kModeHeun && !PACKED && !QUEUE ? 0 : 4;
     return !PACKED && sizeof(R) == 4 && PPT == 2 && MODE == kModeXorshift ? ABP_BLOCKS_XS2 : 0;
 }
 
@@ -774,7 +777,7 @@ __device__ __forceinline__ void zero_hist(uint32_t *sh, const Hist &h) {
 // trajectories.  Packed tiles: blocks of any width w, each taking PPT w consecutive
 // trajectories.
 template <typename R, int PPT, bool PACKED, int MODE>
-__global__ void __launch_bounds__(PACKED ? kThreads / PPT : kThreads, (min_blocks<R, PPT, MODE, PACKED>()))
+__global__ void __launch_bounds__(PACKED ? kThreads / PPT : kThreads, (min_blocks<R, PPT, MODE, PACKED, false>()))
     integrate_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp, int64_t g0, int64_t g1) {
     extern __shared__ uint32_t sh[];
     if constexpr (!PACKED) zero_hist(sh, h);
@@ -943,8 +946,9 @@ __device__ __forceinline__ void store_release(int32_t *p, int v) {
 // bounded: past q.wait_limit_ns the block records status 1 and every block
 // leaves at its next check, without touching the item.
 template <typename R, int PPT, int MODE>
-__global__ void __launch_bounds__(kThreads, (min_blocks<R, PPT, MODE>())) persistent_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp,
-                                                      Queue q, int64_t g0, int64_t g1, int64_t seg) {
+__global__ void __launch_bounds__(kThreads, (min_blocks<R, PPT, MODE, false, true>()))
+    persistent_kernel(Batch b, State st, Hist h, Ckpt ck, Noise nz, KeyParam kp, Queue q, int64_t g0, int64_t g1,
+                      int64_t seg) {
     extern __shared__ uint32_t sh[];
     __shared__ int s_tile, s_round;
     zero_hist(sh, h);
