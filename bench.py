@@ -8,7 +8,9 @@ accumulation, v0 ~ N(0, sqrt(D)), Philox seed 1.  One step of the benchmark is o
 of the whole path: initial condition, integration with noise generation, the final
 histogram of x mod L and the FP64 ensemble reduction.
 
-Prints one JSON line (rank 0).  ``--impl reference`` times the FP64 CPU oracle instead.
+Prints one JSON line (rank 0): the headline with one number per other leg; the legs' full
+records go to stderr as a JSON line of their own, or with ``--detail FILE`` into that file.
+``--impl reference`` times the FP64 CPU oracle instead.
 """
 from __future__ import annotations
 
@@ -61,6 +63,7 @@ def parse():
     ap.add_argument("--small", action="store_true",
                     help="the sweep grid at 2,000 steps (profiling and quick checks; not a bench line)")
     ap.add_argument("--no-adjoint", action="store_true", help="skip the pathwise-adjoint leg")
+    ap.add_argument("--detail", default="", help="file for the full records of the other legs (default: stderr)")
     ap.add_argument("--no-visualisation", action="store_true",
                     help="skip the per-cycle cost of reading intermediate results (iterations lost)")
     ap.add_argument("--profile-config", default="",
@@ -673,6 +676,36 @@ def configs_leg(A, stream, names, lane_peak):
     return out
 
 
+# The legs' records in full make a line of some 22 KB; readers that keep the end of the output
+# would lose its beginning, where the headline stands.
+DETAIL_KEYS = ("adjoint", "visualisation", "configs")
+
+
+def headline(line):
+    """The line that is printed: everything but the legs' records, and one number per leg."""
+    out = {k: v for k, v in line.items() if k not in DETAIL_KEYS}
+    legs = {}
+    adj = line.get("adjoint")
+    if adj:
+        legs["adjoint"] = {k: adj[k] for k in ("forward_ms", "backward_ms") if k in adj}
+    for name, r in (line.get("configs") or {}).items():
+        if isinstance(r, dict) and isinstance(r.get("value"), (int, float)):
+            legs[name] = r["value"]
+    if legs:
+        out["legs"] = legs
+    return out
+
+
+def print_line(line, detail=""):
+    rec = {k: line[k] for k in DETAIL_KEYS if line.get(k)}
+    if rec and detail:
+        with open(detail, "w") as f:
+            json.dump(rec, f)
+    elif rec:
+        print(json.dumps({"detail": rec}), file=sys.stderr, flush=True)
+    print(json.dumps(headline(line)), flush=True)
+
+
 # ----------------------------------------------------------------------------- GPU arm
 
 def main():
@@ -871,7 +904,7 @@ def main():
                 "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches, "clocks": clocks,
                 "adjoint": adj, "visualisation": vis, "configs": cfgs,
                 "wall_s_timed": wall, "sm_count": n_sm, "device": props.name}
-        print(json.dumps(line), flush=True)
+        print_line(line, args.detail)
     ens.close()
     if dist is not None:
         dist.destroy_process_group()
