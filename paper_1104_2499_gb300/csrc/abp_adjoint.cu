@@ -964,14 +964,19 @@ bool use_states(const abp_ctx *ctx, int64_t n_seg, double budget) {
 }
 
 // Segments per launch: as many as this many bytes of buffers hold (one where a segment's
-// own buffers are larger, or the noise is drawn again), shared evenly over the launches.  A launch and its events cost
-// the host some 5 us and the device the start and the drain of its blocks, and level 1 of
-// several segments runs side by side: with short segments of small batches that is most
-// of the time.  Backward, one segment per launch against 128 MB: 19,684 trajectories x
-// 3,029 steps, K = 64, 894 -> 647 us; 8,000 x 2,000, K = 64, 497 -> 327; 256 x 4,000,
-// K = 64, 855 -> 479; 8,000 x 2,000, K = 333, 320 -> 303.  64 MB: 694, 426, 484, 313;
-// 256 MB: 625, 321, 477, 308.  A segment of 262,144 trajectories and K = 333 to 1,000 fills
-// the GPU and the buffers by itself.
+// own buffers are larger, or the noise is drawn again), shared evenly over the launches.  A
+// launch and its events cost the host some 5 us and the device the start and the drain of
+// its blocks, and level 1 of several segments runs side by side: with short segments of
+// small batches that is most of the time.  Backward with the hand-off over 4,000 steps, one
+// segment per launch against as many as fit: 256 trajectories, K = 64, 892 -> 455 us, K = 200,
+// 515 -> 400; 40,000, K = 64, 1,137 -> 884; 60,000 1,315 -> 1,114.  A segment of 262,144
+// trajectories and K = 333 to 1,000 fills the GPU and the buffers by itself.
+// Level 1 of the next launch runs beside the sweep: while the batch is small enough for both
+// to have their warps (of 64 trajectories) on schedulers of their own, no more segments than
+// leave them that.  Past it a sweep that shares its scheduler holds up the launch: 4,000
+// trajectories, K = 64, eight segments 519 us, twelve 768; 8,000, K = 200, three 458, five
+// 660; 12,000 two 481, four 730; 16,384 one 522, two 777; 24,576 one 699, two 929.  At 32,768
+// and more the schedulers are shared either way (K = 64, one 1,227, four 775).
 #ifndef ABP_ADJ_LAUNCH_BYTES
 #define ABP_ADJ_LAUNCH_BYTES (128 << 20)
 #endif
@@ -982,6 +987,9 @@ int64_t segments_per_launch(const abp_ctx *ctx, bool words, bool states, double 
                             (double)std::max<size_t>(L.sub + L.words, 1));
     if (words) per = std::min(per, (int64_t)(budget / (double)std::max<size_t>(L.words, 1)));
     if (states) per = std::min(per, (int64_t)(budget / (double)std::max<size_t>(L.sub, 1)));
+    const int64_t lone = (int64_t)4 * 64 * ctx->sm_count;  // trajectories of one warp per scheduler
+    if (words && 3 * ctx->total_traj <= 2 * lone)
+        per = std::min(per, lone / std::max<int64_t>(ctx->total_traj, 1) - 1);
     per = std::max<int64_t>(1, std::min({per, n_seg, (int64_t)65535}));
     const int64_t launches = (n_seg + per - 1) / per;
     return launches > 0 ? (n_seg + launches - 1) / launches : 1;

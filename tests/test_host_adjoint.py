@@ -256,3 +256,17 @@ assert (L.fake_streams() - streams, L.fake_events() - events) == (1 + 3, 6 + 10)
 A.abp_destroy(ctx)
 assert (L.fake_streams() - streams, L.fake_events() - events) == (1, 6)
 '''.replace("STEP", str(step_bytes)), **form)
+
+
+# segments per launch with the hand-off, 152 SMs: level 1 of the next launch and the sweep each keep
+# to schedulers of their own ((per + 1) T <= 38,912) while T <= 25,941; beyond, and for tiny
+# batches, all ten segments at once
+@pytest.mark.parametrize("n_traj,launches", [(100, 1), (3500, 1), (4000, 2), (8000, 4), (12000, 5), (16384, 10),
+                                             (25941, 10), (25942, 1)])
+def test_handoff_launches_leave_the_sweep_its_schedulers(child, n_traj, launches):
+    child('''
+ctx, grad, dv = integrated(n_traj=(N,), n_steps=(400,), K=40)
+n0 = L.fake_launches()
+A.abp_backward(ctx, None, grad)
+assert sum("reverse_pair" in k for k in kernels(n0)) == COUNT, kernels(n0)
+'''.replace("(N,)", "(%d,)" % n_traj).replace("COUNT", str(launches)), ABP_ADJ_STATE_BYTES="0")
