@@ -56,10 +56,10 @@ static_assert(kSub % 4 == 0 && (kBlockSteps % kSub) == 0, "sub-chunks hold whole
 
 // Sub-chunks lie on absolute multiples of kSub steps (not on offsets from the segment's
 // start, where a checkpoint interval that is no multiple of kSub sent every chunk of most
-// segments down the one-step-at-a-time path: 262,144 trajectories x 4,000 steps, forward
-// and backward, K = 500 5.93 -> 3.98 ms, K = 333 7.60 -> 4.21 ms), so that a whole chunk holds whole
-// Philox blocks and no position fold falls inside it whatever the segment's start: the
-// segment [s0, s1) has chunks c0 = s0 / kSub .. (s1 - 1) / kSub, the first and the last
+// segments down the one-step-at-a-time path, without the hand-off: backward of 262,144
+// trajectories x 4,000 steps, K = 500 5.2 ms then and 2.66 now, K = 333 6.7 and 2.83, K =
+// 1,000 2.82 and 2.59), so that a whole chunk holds whole Philox blocks and no position
+// fold falls inside it whatever the segment's start: the segment [s0, s1) has chunks c0 = s0 / kSub .. (s1 - 1) / kSub, the first and the last
 // of them possibly partial (when checkpoint_every or the run's length is not a multiple
 // of kSub).
 struct SegChunks {
@@ -217,14 +217,6 @@ __device__ __forceinline__ void block_sum6(double (&a)[6], double (*red)[6]) {
     }
 }
 
-// Level 1 of segment [s0, s1) of two trajectories (idx[0], idx[1]) of one thread: re-run
-// from their checkpoints c0, c1, leaving the state at the start of each chunk in the
-// sub-checkpoint scratch.  Whole
-// chunks step the pair with paired FP32 instructions (same operations
-// as em_step_f32 / box_muller_f32 on each half, so the sub-checkpoints are the
-// scalar ones bit for bit); other chunks step each trajectory on its own.
-// store1: whether the second trajectory is real (else it duplicates the first
-// one's neighbour and its sub-checkpoints are not written).
 // One Philox block of the hand-off for the thread's two trajectories: the
 // scaled Box-Muller radii of its two word pairs (nrA, nrB, as their bits) and
 // the two angle words, (nrA, wb_A, nrB, wb_B).  The buffer is laid out by
@@ -256,6 +248,13 @@ __device__ __forceinline__ void pair_blocks(uint32_t m, const StepStream (&ss)[2
     w1 = step_block(SHARED ? h0 : block_head(m, ss[1].hx), ss[1], K);
 }
 
+// Level 1 of segment [s0, s1) of two trajectories (idx[0], idx[1]) of one thread: re-run
+// from their checkpoints c0, c1, leaving the state at the start of each chunk in the
+// sub-checkpoint scratch.  Whole chunks step the pair with paired FP32 instructions (same
+// operations as em_step_f32 / box_muller_f32 on each half, so the sub-checkpoints are the
+// scalar ones bit for bit); other chunks step each trajectory on its own.
+// store1: whether the second trajectory is real (else it duplicates the first
+// one's neighbour and its sub-checkpoints are not written).
 template <bool WORDS>
 __device__ __forceinline__ void level1_segment2(const AdjArgs &a, float4 *slots, uint4 *wp, const Coef<float> &k,
                                                 const StepStream (&ss)[2], const int64_t (&idx)[2], bool store1,
@@ -683,7 +682,7 @@ __global__ void __launch_bounds__(kL1Threads) adjoint_states_kernel(AdjArgs a, i
 // their sines wait for shared memory, so longer groups are faster as long as the ring leaves
 // room for six warps on an SM (32 KB each): backward of 256 trajectories x 4,000 steps, K =
 // 64, 262 us with eight groups of 8, 235 with four of 16, 237 with three; of 16,384 x 4,000,
-// K = 200, 480, 468 and 516 us.
+// K = 200, 480, 468 and 516 us (each some 20 us less since the calls ask for no free memory).
 constexpr int kRowGroup = 16, kRowGroups = 4, kSweepThreads = 32;
 
 __global__ void __launch_bounds__(kSweepThreads) adjoint_sweep_kernel(AdjArgs a, SegView sv, int64_t seg0, int n,
@@ -939,13 +938,14 @@ double handoff_memory(const abp_ctx *ctx) {
 
 // Whether level 1 hands every step's state to the sweep (adjoint_states_kernel): batches of
 // at most kStateTraj trajectories whose segments fit ABP_ADJ_STATE_BYTES (0: never) and
-// the hand-off's budget.  Backward of the pair kernels against this: 256 trajectories x
-// 4,000 steps, K = 64, 482 -> 235 us; 8,000 x 2,000, K = 64, 333 -> 199, K = 333, 309 ->
-// 202; 8,192 x 4,000, K = 1,000, 487 -> 302; 16,384 x 4,000, K = 200, 869 -> 468; 24,576 x
-// 4,000, K = 1,000, 625 -> 600; 32,768 x 2,000, K = 64, 588 -> 491: beyond that the SMs
-// hold more warps than the ring leaves room for and the rows' 32 bytes a step come from
-// HBM.  Fewer bytes mean more launches (with groups of 8 rows and 512 MB 206, 210 and 319
-// us for the second to fourth of these, 256 MB 217, 212 and 369, 128 MB 249, 240 and 488).
+// the hand-off's budget.  One backward, the hand-off against this: 300 trajectories x 4,000
+// steps, K = 64, 458 -> 205 us; 8,000 x 2,000, K = 64, 341 -> 170, K = 333, 281 -> 174; 8,000
+// x 4,000, K = 1,000, 446 -> 275; 16,384 x 4,000, K = 200, 521 -> 440; 24,576 x 4,000, K = 64,
+// 966 -> 636 (K = 500, one segment per launch, 647 and 706); 32,768 x 2,000, K = 64, 475 ->
+// 465: beyond that the SMs hold more warps than the ring leaves room for and the rows' 32
+// bytes a step come from HBM.  Fewer bytes mean more launches (256 MB: 8,000 x 2,000 182 and
+// 211 us, 16,384 x 4,000 508; 128 MB: 209, 215 and 647), more cost an allocation and its
+// release: up to 0.1 ms of a context's first call and 0.2 of its end at 512 MB.
 #ifndef ABP_ADJ_STATE_TRAJ
 #define ABP_ADJ_STATE_TRAJ 32768
 #endif
@@ -1275,6 +1275,7 @@ extern "C" abp_status abp_backward_traj(abp_ctx *ctx, double *dvbar) {
     a.sub = nullptr;
     a.n_sub = n_sub;
     a.words = nullptr;
+    a.per = 1;
     a.tile0 = 0;
     a.n_blk = 0;
     a.w = nullptr;
