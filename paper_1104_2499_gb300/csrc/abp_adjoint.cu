@@ -1137,8 +1137,12 @@ extern "C" abp_status abp_backward_windowed(abp_ctx *ctx, const double *dJ_dmean
         // 262,144 trajectories 2.67 -> 2.48 ps per particle-step, 175,104 2.91 -> 2.56,
         // 131,072 3.09 -> 2.71, 1,048,576 2.40 -> 2.38 (three, four and six groups: within 2%
         // of two).  A batch with fewer blocks than SMs runs in one group: it leaves SMs
-        // free anyway, and each launch costs host time.
-        const int n_grp = !states && ctx->n_tiles >= 2 && (int64_t)ctx->n_tiles * sub2 >= ctx->sm_count ? kAdjGroups : 1;
+        // free anyway, and each launch costs host time.  With one or two launches there is
+        // little to fill in, so one group too unless it has three blocks per SM (K = 1,000, 2,000
+        // steps, two groups against one: 50,000 trajectories 495 us and 430, 100,000 702 and
+        // 662, 131,072 793 and 858, 262,144 1,377 and 1,418).
+        const int64_t blocks = (int64_t)ctx->n_tiles * sub2;
+        const int n_grp = !states && ctx->n_tiles >= 2 && blocks >= (n_run > 2 ? 1 : 3) * (int64_t)ctx->sm_count ? kAdjGroups : 1;
         // the groups' streams and events, kept for the next call
         for (int i = 0; e == cudaSuccess && i < 2 * n_grp - 1; ++i)
             if (!ctx->adj_stream[i]) e = cudaStreamCreateWithFlags(&ctx->adj_stream[i], cudaStreamNonBlocking);

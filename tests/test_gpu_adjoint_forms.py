@@ -118,11 +118,15 @@ def test_trajectories_match_the_oracle(abp, form, K, window, name):
         np.testing.assert_allclose(mine.mean(axis=0), g[i], rtol=1e-9, atol=1e-12 * np.abs(g[i]).max())
 
 
-# Two groups of tiles (as many blocks of the paired sweep as SMs): 93 tiles of 512, odd and ragged,
-# several launches, twice on one context, against the same trajectories set by set, which run as one
-# group.  The hand-off for all, for one segment at a time (K = 50: 8 slots of 8 steps, 2 blocks of
-# noise each, in 93 x 2 kernel blocks) and not at all.
-@pytest.mark.parametrize("handoff", ["", str(2 * 16 * 93 * 2 * 8 * 2 * 2 * 128 + 4096), "0"], ids=["all", "one", "none"])
+# Two groups of tiles (as many blocks of the paired sweep as SMs and more than two launches): 93
+# tiles of 512, odd and ragged, twice on one context, against the same trajectories set by set,
+# which run as one group.  The hand-off for all (one group), for one and for two segments at a time
+# (8 slots of 8 steps, 2 blocks of noise each, in 93 x 2 kernel blocks) and not at all.
+SEGMENT = 2 * 16 * 93 * 2 * 8 * 2 * 2 * 128
+
+
+@pytest.mark.parametrize("handoff", ["", str(SEGMENT + 4096), str(2 * SEGMENT + 4096), "0"],
+                         ids=["all", "one", "two", "none"])
 @pytest.mark.parametrize("K,window", [(50, 0), (50, 100), (64, 0)])
 def test_two_groups_match_one(abp, form, monkeypatch, K, window, handoff):
     form("handoff")

@@ -270,3 +270,17 @@ n0 = L.fake_launches()
 A.abp_backward(ctx, None, grad)
 assert sum("reverse_pair" in k for k in kernels(n0)) == COUNT, kernels(n0)
 '''.replace("(N,)", "(%d,)" % n_traj).replace("COUNT", str(launches)), ABP_ADJ_STATE_BYTES="0")
+
+
+# two groups of tiles: as many blocks of the paired sweep as SMs, and more than two launches or
+# three times as many
+@pytest.mark.parametrize("n_traj,K,groups", [(38000, 20, 1), (39000, 20, 2), (39000, 200, 1), (116000, 200, 1),
+                                             (117000, 200, 2)])
+def test_groups_of_tiles(child, n_traj, K, groups):
+    child('''
+ctx, grad, dv = integrated(n_traj=(N,), n_steps=(400,), K=KK)
+n0, streams = L.fake_launches(), L.fake_streams()
+A.abp_backward(ctx, None, grad)
+assert L.fake_streams() - streams == (1 if GROUPS == 1 else 3), kernels(n0)
+'''.replace("(N,)", "(%d,)" % n_traj).replace("KK", str(K)).replace("GROUPS", str(groups)),
+          ABP_ADJ_HANDOFF_BYTES="0")
