@@ -862,7 +862,11 @@ __device__ __forceinline__ void ws_produce(const Batch &b, const State &st, cons
                 out[i * 32] = make_float2(nr, cs);
             }
         } else if constexpr (sizeof(R) == 8) {
-            for (int j = p; j < SS / 4; j += NP) {
+            // only the blocks the launch steps through: an FP64 transform takes a microsecond
+            // (4,096 trajectories, windows of 7 steps: 15.6 us each against 38 with whole slots)
+            const int j0 = (int)(max(n_begin - a * SS, (int64_t)0) >> 2);
+            const int j1 = (int)((min(n_end - a * SS, (int64_t)SS) + 3) >> 2);
+            for (int j = j0 + p; j < j1; j += NP) {
                 const uint4 wv = step_block((uint32_t)(a * (SS / 4) + j), ss, K);
                 double z[4];
                 box_muller_step_f64(wv.x, wv.y, z[0], z[1]);
@@ -1320,8 +1324,13 @@ cudaError_t launch_integrate_t(const Batch &b, const State &s, const Hist &h, co
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
+    // FP64, a window of one step (a caller that looks at every step): the one normal drawn by
+    // the stepping thread itself takes less than a counter block and its hand-over (4,096
+    // trajectories 8.7 us a window against 10.7); from two steps on the producers are ahead
+    // (two 10.7 us against 12.8, seven 15.6 against 25.3).
+    const int64_t steps = g1 - g0;
     if constexpr (PPT == 1 && ABP_WS) {
-        if (b.narrow > 0 && b.narrow <= ABP_WS_WIDEST && wait && wait->status) {
+        if (b.narrow > 0 && b.narrow <= ABP_WS_WIDEST && wait && wait->status && !(sizeof(R) == 8 && steps < 2)) {
             bool taken = false;
             const cudaError_t e = launch_ws<R, MODE>(b, s, h, c, nz, g0, g1, *wait, st, taken);
             if (e != cudaSuccess || taken) return e;
