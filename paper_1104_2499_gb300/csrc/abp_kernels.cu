@@ -1342,15 +1342,19 @@ cudaError_t launch_integrate_t(const Batch &b, const State &s, const Hist &h, co
     if (b.n_single > 0)
         kern<<<(unsigned)(b.n_single * sub_s), threads, smem, st>>>(b, s, h, c, nz, key_param(nz.k0, nz.k1), g0, g1);
     if (n_packed > 0) {  // histograms in global memory
-        const int w = b.packed_threads;
-        const unsigned grid = n_packed * (unsigned)(kThreads / (w * b.packed_ppt));
+        // A window of a few steps is bound by its launch and loads, and two trajectories per
+        // thread load a set each: one per thread up to 8 steps (a window of one step, 250 tiles
+        // 5.7 us against 7.5; of two, 1,000 tiles 10.0 and 11.8; of four, 250 tiles 6.8 and 7.8;
+        // of eight 8.8 and 8.8; of 20 the pairs are ahead: 1,000 tiles 17.0 against 17.6).
+        const int ppt = steps <= 8 ? 1 : b.packed_ppt, w = b.packed_ppt != ppt ? kThreads : b.packed_threads;
+        const unsigned grid = n_packed * (unsigned)(kThreads / (w * ppt));
         const KeyParam kp = key_param(nz.k0, nz.k1);
         bool paired = false;
         if constexpr (sizeof(R) == 4 && MODE != kModeXorshift) {
-            paired = b.packed_ppt == 2;
+            paired = ppt == 2;
             if (paired) integrate_kernel<R, 2, true, MODE><<<grid, w, 0, st>>>(b, s, h, c, nz, kp, g0, g1);
         }
-        if (!paired && b.packed_ppt != 1) return cudaErrorInvalidValue;
+        if (!paired && ppt != 1) return cudaErrorInvalidValue;
         if (!paired) integrate_kernel<R, 1, true, MODE><<<grid, w, 0, st>>>(b, s, h, c, nz, kp, g0, g1);
     }
     return cudaGetLastError();

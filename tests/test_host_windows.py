@@ -1,5 +1,6 @@
 """Which integrator a window launches, on the CPU (tests/helpers/fake_cudart.cpp): windows of one
-step take the plain kernel where the FP64 state is otherwise warp-specialised."""
+step take the plain kernel where the FP64 state is otherwise warp-specialised, windows of up to
+eight steps one trajectory per thread where packed tiles otherwise hold two."""
 import pytest
 
 from test_host_adjoint import child  # noqa: F401  (the library linked with the fake runtime)
@@ -22,6 +23,10 @@ for ks, want in zip(got, WANT):
     (1, 4096, {}, True, "integrate_kernelIdLi1ELb0", "ws_kernelIdLb0", "ws_kernelIdLb0"),
     (70, 1, {}, True, "integrate_kernelIdLi1ELb1", "ws_kernelIdLb1", "ws_kernelIdLb1"),
     (1, 4096, {}, False, "ws_kernelIfLb0", "ws_kernelIfLb0", "ws_kernelIfLb0"),
+    (3000, 20, {}, False, "integrate_kernelIfLi1ELb1", "integrate_kernelIfLi1ELb1",
+     "integrate_kernelIfLi2ELb1"),
+    (3000, 20, {"scheme": 1}, False, "integrate_kernelIfLi1ELb1", "integrate_kernelIfLi1ELb1",
+     "integrate_kernelIfLi2ELb1"),
     (3000, 20, {"noise": 1}, False, "integrate_kernelIfLi1ELb1", "integrate_kernelIfLi1ELb1",
      "integrate_kernelIfLi1ELb1"),
     (3000, 20, {}, True, "integrate_kernelIdLi1ELb1", "integrate_kernelIdLi1ELb1",
